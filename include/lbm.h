@@ -242,8 +242,12 @@ int lbm_get_layout(const lbm_ctx* ctx, int* pitch, int* grid, int* block);
  *                    segments into a ring of `stages` (2-4; 0 = default) shared-memory stages
  *                    on mbarriers while 4-16 consumer warps (lbm_set_tile_form) collide
  *                    earlier tiles; needs nx * (bytes per population) to be a multiple of 16.
- *   LBM_PATH_AUTO    BULK where the row length allows it and a time step has at least one
- *                    tile per resident CTA, else VECTOR (the default).
+ *   LBM_PATH_AUTO    (the default) runs of two or more steps of 32- or 16-bit lattices with the
+ *                    extended equilibrium take time-fused launches, each of which advances up to
+ *                    four steps with one read and one write of the populations (unless stages, a
+ *                    launch shape or a tile form is asked for); every other step BULK where the
+ *                    row length allows it and a time step has at least one tile per resident CTA,
+ *                    else VECTOR.  The arithmetic of a node is the same, bit for bit.
  * Applies to the context's next lbm_step and to groups created afterwards.  Errors:
  * LBM_ERR_INVALID_ARG for an unknown path or stage count, LBM_ERR_UNSUPPORTED for BULK on a
  * lattice whose rows are not a multiple of 16 bytes. */
@@ -311,7 +315,8 @@ void lbm_group_destroy(lbm_group* g);
  * launch per time step; otherwise each context gets its own launch. */
 int lbm_group_set_timing(lbm_group* g, int enable);
 int lbm_group_timing(lbm_group* g, double* replay_ms, long long* lattice_steps, long long* kernel_launches);
-/* How the group is advanced (library design choice; the paper has no counterpart): *family =
+/* How the group is advanced a step at a time (library design choice; the paper has no counterpart;
+ * runs of several steps may take the time-fused launches of LBM_PATH_AUTO instead): *family =
  * LBM_PATH_BULK (copy-engine staged launches over all contexts), or LBM_PATH_VECTOR
  * (register-staged: one multi-lattice launch per step, or one launch per context and step);
  * for LBM_PATH_BULK, *form = LBM_FORM_GENERAL / LBM_FORM_LIGHT / LBM_FORM_WIDE, *steps_per_launch

@@ -13,6 +13,7 @@
 #include "lbm.h"
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
+#include "lbm_march.cuh"
 #include "lbm_tile.cuh"
 
 using lbm::CheckArgs;
@@ -74,15 +75,22 @@ struct lbm_group {
     int same_geometry = 0;             // every context has the same units and tiles per unit
     int wU = 0, wntx = 0;              // that geometry
     long long state_bytes = 0;         // both buffers of every context
+    int march = 0;                     // most time steps of a time-fused launch, 0 = none
+    const void* mkernel[2] = {nullptr, nullptr};   // default shift / reference-velocity shift
+    int mgrid = 0;                     // their resident CTAs (of kMarchWarps warps)
+    int msmem = 0;                     // their shared memory per warp
+    int mixed = 0;                     // contexts of several models
     cudaStream_t stream = nullptr;
     cudaStream_t capture = nullptr;
     std::vector<cudaStream_t> side;    // concurrent blow-up checks (launch_checks)
     std::vector<cudaEvent_t> side_done;
     cudaEvent_t fork = nullptr;
     int graph_steps = 0;
-    cudaGraphExec_t exec = nullptr;
-    std::vector<int> exec_parity;      // ctx->cur of each context when the graph was recorded
-    std::vector<unsigned> exec_gen;    // ctx->gen of each context when the graph was recorded
+    struct Recorded {                  // a recorded graph, by the parity of the first context's buffer
+        cudaGraphExec_t exec = nullptr;
+        std::vector<int> parity;       // ctx->cur of each context when the graph was recorded
+        std::vector<unsigned> gen;     // ctx->gen of each context when the graph was recorded
+    } rec[2];
     int timing = 0;
     std::vector<cudaEvent_t> ev;       // pairs (start, stop) of timed replays
     size_t ev_used = 0;
@@ -199,6 +207,22 @@ bool pick_tile_kernel(int storage, bool shifted, int stages, int form, lbm::Tile
         case LBM_BF16: return lbm::tile_kernel_bf16(shifted, stages, form, out);
         default: return false;
     }
+}
+const void* pick_march_kernel(int storage, bool shifted, bool pairs, bool roll) {
+    switch (storage) {
+        case LBM_F32: return lbm::march_kernel_f32(shifted, pairs, roll);
+        case LBM_F16: return lbm::march_kernel_f16(shifted, pairs, roll);
+        case LBM_BF16: return lbm::march_kernel_bf16(shifted, pairs, roll);
+        default: return nullptr;
+    }
+}
+// shared memory of one warp of the time-fused kernel, and its most time steps of a launch
+int march_smem(int storage, bool roll) {
+    if (storage == LBM_F32) return roll ? lbm::march_smem_bytes<float, true> : lbm::march_smem_bytes<float, false>;
+    return roll ? lbm::march_smem_bytes<__half, true> : lbm::march_smem_bytes<__half, false>;
+}
+int march_most(int storage) {
+    return storage == LBM_F32 ? lbm::MarchForm<float>::TMAX : lbm::MarchForm<__half>::TMAX;
 }
 // the light kernel form (float, half, bfloat16) serves groups whose lattices all run BGK, RM,
 // HM or PR
@@ -449,9 +473,134 @@ int tile_steps_per_launch(const lbm_group* g) {
     return (int)std::min<long long>(std::min<long long>(per, cap), LBM_TILE_STEPS_PER_LAUNCH);
 }
 
-// n time steps of the group: bulk-copy launches for a tiled group, else n launches
-int group_advance(lbm_group* g, cudaStream_t s, long long n) {
+// FP32 operations of one node update, by model (lbm_device.cuh)
+int march_cost(int model) {
+    static const int cost[] = {60, 66, 68, 79, 81, 85, 65, 75};
+    return cost[kernel_model(model)];
+}
+
+// Strips x rows of the group's lattices when t steps are fused.
+long long march_strip_rows(const lbm_group* g, int t) {
+    const int width = lbm::march_width(t);
+    long long rows = 0;
+    for (const lbm_ctx* c : g->ctx) rows += (long long)((c->nx + width - 1) / width) * c->ny;
+    return rows;
+}
+
+// How a run is fused: steps per launch and marches (warps) per launch.
+struct MarchPlan {
+    int t;
+    long long warps;
+};
+
+// Large lattices fuse as many steps as the kernel has levels, in whole waves of resident warps
+// that march 80-160 rows: shorter, and the t - 1 rows each level recomputes weigh; longer, and
+// neighbouring marches drift apart and lose each other's lines (16384^2 FP32 K against 128 rows:
+// 32 rows 1.08x the time, 64 1.03x, 256 1.02x, one wave 1.05x).  Mixed models take at least two
+// waves, which level out SMs of unequal work (eight 1024^2 lattices 0.98x).
+// Small lattices trade launches against redundant rows: the plan with the least time by a model of
+// what was measured on 67 x 37 to 1024^2 lattices -- a launch takes 2.2 us and its longest march,
+// t (H + t - 1) level-rows for H rows, at 0.21 us a level-row with a scheduler to itself, more with
+// company up to 0.42 + 0.5 / t when every slot is taken (512^2, us a step: t = 2 2.9, 3 3.2, 4 3.6;
+// 256^2: t = 4 on 304 warps 2.0, on 640 2.2; 128^2: 1.5 on 192, 1.9 on 96).
+MarchPlan march_plan(const lbm_group* g, long long n) {
+    const long long slots = (long long)g->mgrid * lbm::kMarchWarps, scheds = slots / 4;
+    const int most = (int)std::min<long long>(g->march, n);
+    const long long rows = march_strip_rows(g, most);
+    if (most == g->march && rows >= 24 * slots) {
+        long long waves = (rows + 160 * slots - 1) / (160 * slots);
+        if (g->mixed && waves < 2 && rows >= 48 * slots) waves = 2;
+        return {most, slots * waves};
+    }
+    MarchPlan best{most, 1};
+    double least = 1e300;
+    for (int t = 2; t <= most; ++t) {
+        const long long r = march_strip_rows(g, t);
+        for (long long w = scheds / 2; w <= slots; w *= 2) {
+            const long long warps = std::max<long long>(1, std::min(w, r / 2));   // two rows at least
+            const double load = (double)warps / scheds, height = (double)r / warps;
+            const double each = load <= 0.5 ? 0.21 : std::min(0.42 + 0.5 / t, 0.2 + 0.15 * load);
+            const double us = (2.2 + each * t * (height + t - 1)) / t;
+            if (us < least) {
+                least = us;
+                best = {t, warps};
+            }
+        }
+    }
+    return best;
+}
+
+// Whether a run of n steps takes the time-fused launches (at least two steps: a single one is
+// what the one-step kernels are for).
+bool use_march(const lbm_group* g, long long n) { return g->march > 1 && n >= 2 && tile_shift(g) >= 0; }
+
+// Time-fused launches of a run of n steps, t at most in each; `even` (a recorded graph, which must
+// end on the buffers it began with) one more if that is odd.
+long long march_launches(long long n, int t, bool even) {
+    const long long l = (n + t - 1) / t;
+    return even && l % 2 ? l + 1 : l;
+}
+
+// One time-fused launch: t time steps of every context on about `warps` warps.
+int launch_march(lbm_group* g, cudaStream_t s, int t, long long warps) {
+    lbm::MarchArgs ma;
+    ma.n = (int)g->ctx.size();
+    ma.t = t;
+    const int width = lbm::march_width(t);
+    double work = 0.0;
+    for (const lbm_ctx* c : g->ctx) work += (double)((c->nx + width - 1) / width) * c->ny * march_cost(c->model);
+    // few warps go to as many SMs as there are; full CTAs keep neighbouring strips together
+    const int per = warps < (long long)g->mgrid * lbm::kMarchWarps ? 2 : lbm::kMarchWarps;
+    unsigned begin = 0;
+    for (size_t k = 0; k < g->ctx.size(); ++k) {
+        lbm_ctx* c = g->ctx[k];
+        lbm::MarchEntry& e = ma.e[k];
+        e.src = c->buf[c->cur];
+        e.dst = c->buf[c->cur ^ 1];
+        e.plane = c->plane;
+        e.nx = c->nx; e.ny = c->ny; e.pitch = c->pitch;
+        e.model = kernel_model(c->model);
+        e.strips = (c->nx + width - 1) / width;
+        // bands by the lattice's share of the work, so that every march costs about the same
+        const double bands = (double)warps * c->ny * march_cost(c->model) / work;
+        e.bands = std::max(1, std::min(c->ny, (int)bands));
+        e.begin = begin;
+        begin += (unsigned)((e.strips * (long long)e.bands + per - 1) / per);
+        const StepArgs a = step_args(c);
+        for (int j = 0; j < lbm::kNumConsts; ++j) e.c[j] = make_float2(a.cf[j], a.cf[j]);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(begin);
+    cfg.blockDim = dim3(32 * per);
+    cfg.dynamicSmemBytes = (size_t)(g->msmem * per);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[] = {(void*)&ma};
+    LBM_CK(g->ctx[0], cudaLaunchKernelExC(&cfg, g->mkernel[tile_shift(g)], args));
+    for (lbm_ctx* c : g->ctx) {
+        c->cur ^= 1;
+        c->steps += t;
+    }
+    return LBM_OK;
+}
+
+// n time steps of the group: time-fused launches where the group has them, else bulk-copy
+// launches for a tiled group, else n launches
+int group_advance(lbm_group* g, cudaStream_t s, long long n, bool even = false) {
     if (n <= 0) return LBM_OK;
+    if (use_march(g, n)) {
+        const MarchPlan p = march_plan(g, n);
+        const long long l = march_launches(n, p.t, even);
+        for (long long k = 0; k < l; ++k) {   // lengths differ by at most one step
+            int rc = launch_march(g, s, (int)(n / l + (k < n % l ? 1 : 0)), p.warps);
+            if (rc != LBM_OK) return rc;
+        }
+        return LBM_OK;
+    }
     if (g->tiled && tile_shift(g) >= 0) {
         const int per = tile_steps_per_launch(g);
         for (long long done = 0; done < n;) {
@@ -539,18 +688,19 @@ int launch_checks(lbm_group* g, const std::vector<lbm_ctx*>& due) {
 
 int group_record(lbm_group* g) {
     lbm_ctx* c0 = g->ctx[0];
-    if (g->exec) {
-        cudaGraphExecDestroy(g->exec);
-        g->exec = nullptr;
+    lbm_group::Recorded& R = g->rec[c0->cur];
+    if (R.exec) {
+        cudaGraphExecDestroy(R.exec);
+        R.exec = nullptr;
     }
-    // record on the private stream; the buffers alternate, so after an even number of steps
+    // record on the private stream; the buffers alternate, so after an even number of launches
     // every context is back on the buffer it started from and the graph can be replayed
     std::vector<int> cur0(g->ctx.size());
     std::vector<long long> steps0(g->ctx.size());
     for (size_t k = 0; k < g->ctx.size(); ++k) { cur0[k] = g->ctx[k]->cur; steps0[k] = g->ctx[k]->steps; }
     LBM_CK(c0, cudaStreamBeginCapture(g->capture, cudaStreamCaptureModeThreadLocal));
     int rc = LBM_OK;
-    rc = group_advance(g, g->capture, g->graph_steps);
+    rc = group_advance(g, g->capture, g->graph_steps, true);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(g->capture, &graph);
     for (size_t k = 0; k < g->ctx.size(); ++k) { g->ctx[k]->cur = cur0[k]; g->ctx[k]->steps = steps0[k]; }
@@ -559,23 +709,24 @@ int group_record(lbm_group* g) {
         return rc;
     }
     if (e != cudaSuccess) return set_err(c0, LBM_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&g->exec, graph, 0);
+    e = cudaGraphInstantiate(&R.exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
-        g->exec = nullptr;
+        R.exec = nullptr;
         return set_err(c0, LBM_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
     }
-    g->exec_parity = cur0;
-    g->exec_gen.resize(g->ctx.size());
-    for (size_t k = 0; k < g->ctx.size(); ++k) g->exec_gen[k] = g->ctx[k]->gen;
+    R.parity = cur0;
+    R.gen.resize(g->ctx.size());
+    for (size_t k = 0; k < g->ctx.size(); ++k) R.gen[k] = g->ctx[k]->gen;
     return LBM_OK;
 }
 
 int group_replay(lbm_group* g) {
     lbm_ctx* c0 = g->ctx[0];
-    bool same = g->exec != nullptr;
+    lbm_group::Recorded& R = g->rec[c0->cur];
+    bool same = R.exec != nullptr;
     for (size_t k = 0; same && k < g->ctx.size(); ++k)
-        same = (g->ctx[k]->cur == g->exec_parity[k]) && (g->ctx[k]->gen == g->exec_gen[k]);
+        same = (g->ctx[k]->cur == R.parity[k]) && (g->ctx[k]->gen == R.gen[k]);
     if (!same) {
         int rc = group_record(g);
         if (rc != LBM_OK) return rc;
@@ -594,11 +745,13 @@ int group_replay(lbm_group* g) {
         g->ev_used += 2;
         LBM_CK(c0, cudaEventRecord(e0, g->stream));
     }
-    LBM_CK(c0, cudaGraphLaunch(g->exec, g->stream));
+    LBM_CK(c0, cudaGraphLaunch(R.exec, g->stream));
     if (g->timing) {
         LBM_CK(c0, cudaEventRecord(e1, g->stream));
         g->pending_lattice_steps += (long long)g->graph_steps * (long long)g->ctx.size();
-        g->pending_kernels += (g->tiled && tile_shift(g) >= 0)
+        g->pending_kernels += use_march(g, g->graph_steps)
+                                  ? march_launches(g->graph_steps, march_plan(g, g->graph_steps).t, true)
+                              : (g->tiled && tile_shift(g) >= 0)
                                   ? (long long)(g->graph_steps + tile_steps_per_launch(g) - 1) / tile_steps_per_launch(g)
                                   : (long long)g->graph_steps * (g->fused ? 1LL : (long long)g->ctx.size());
     }
@@ -1079,6 +1232,42 @@ int lbm_group_create(lbm_group** out, lbm_ctx* const* ctxs, int n, int graph_ste
         }
         g->fused = 1;
     }
+    // time-fused launches: 32- and 16-bit lattices of one storage type with the extended
+    // equilibrium, unless a context asks for a kernel family, form or launch shape.  (FP64 is bound
+    // by its pipe with one step a launch already.)  Groups of several models take the rolled form,
+    // whose code for four models at a time stays in an SM's instruction cache (eight 1024^2
+    // lattices of all models 42 us a step, unrolled 59; one model: 16384^2 K 1068, unrolled 1042)
+    bool march = n <= lbm::kGroupMax && ctxs[0]->storage != LBM_F64;
+    bool pairs = true, mixed = false;
+    for (int k = 0; k < n; ++k) {
+        const lbm_ctx* c = ctxs[k];
+        mixed = mixed || kernel_model(c->model) != kernel_model(ctxs[0]->model);
+        march = march && c->storage == ctxs[0]->storage && c->eq_order == 4 && c->path == LBM_PATH_AUTO &&
+                c->stages == 0 && c->launch_steps == 0 && c->launch_order == LBM_ORDER_AUTO &&
+                c->tile_form == LBM_FORM_AUTO;
+        pairs = pairs && c->nx % 2 == 0;
+    }
+    if (march) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        for (int sh = 0; sh < 2; ++sh) {
+            int per_sm = 0;
+            g->mkernel[sh] = pick_march_kernel(ctxs[0]->storage, sh == 1, pairs, mixed);
+            g->msmem = march_smem(ctxs[0]->storage, mixed);
+            const int smem = g->msmem * lbm::kMarchWarps;
+            if (cudaFuncSetAttribute(g->mkernel[sh], cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, g->mkernel[sh], 32 * lbm::kMarchWarps, smem) != cudaSuccess ||
+                per_sm < 1) {
+                cudaGetLastError();
+                march = false;
+                break;
+            }
+            g->mgrid = sh == 0 ? sms * per_sm : std::min(g->mgrid, sms * per_sm);
+        }
+        if (march) g->march = march_most(ctxs[0]->storage);
+        g->mixed = mixed ? 1 : 0;
+    }
     if (graph_steps > 0) {
         cudaError_t e = cudaStreamCreateWithFlags(&g->capture, cudaStreamNonBlocking);
         if (e != cudaSuccess) {
@@ -1093,7 +1282,8 @@ int lbm_group_create(lbm_group** out, lbm_ctx* const* ctxs, int n, int graph_ste
 void lbm_group_destroy(lbm_group* g) {
     if (!g) return;
     cudaStreamSynchronize(g->stream);
-    if (g->exec) cudaGraphExecDestroy(g->exec);
+    for (auto& r : g->rec)
+        if (r.exec) cudaGraphExecDestroy(r.exec);
     for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
     if (g->capture) cudaStreamDestroy(g->capture);
     for (cudaStream_t st : g->side) cudaStreamDestroy(st);

@@ -45,11 +45,15 @@ __host__ __device__ inline double shift_of(int i, double rho0, double urx, doubl
 
 // Collision constants, computed once on the host in both precisions (kernels then do no
 // FP64 set-up work, which GB300's narrow FP64 pipe would make costly):
-// [w_nu, w3, w4, rho0, urx, ury, Px0, Px+, Px-, Py0, Py+, Py-, urx^2 + cs^2, ury^2 + cs^2,
-//  ka, kb, kappa, dkappa/dw_nu] -- ka, kb the cumulant model's coefficients
-// cs^2 (c4 - kappa), c4 - kappa^2 (c4 = 1 - w4; kappa = 1 - w_nu, 1 or 0 for the
-// post-collision, pre-collision or equilibrium rebuild of K~22, field `kread`).
-constexpr int kNumConsts = 18;
+//  [0-5]   w_nu, w3, w4, rho0, urx, ury
+//  [6-11]  Px0, Px+, Px-, Py0, Py+, Py- (shift factors phi_s(u_ref))
+//  [12-13] urx^2 + cs^2, ury^2 + cs^2
+//  [14-17] ka, kb, kappa, dkappa/dw_nu -- ka, kb the cumulant model's coefficients
+//          cs^2 (c4 - kappa), c4 - kappa^2 (c4 = 1 - w4; kappa = 1 - w_nu, 1 or 0 for the
+//          post-collision, pre-collision or equilibrium rebuild of K~22, field `kread`)
+//  [18-25] combinations the collision uses: -rho0, w - w3, 2 (w3 - w4), w - 2 w3 + w4,
+//          cs^2 (w - w4), w3 - 1, w4 - 1, cs^2 (w - 1); [26-29] -kb, -w, -w3, -w4
+constexpr int kNumConsts = 30;
 
 struct StepArgs {
     int nx, ny;          // lattice size
@@ -77,11 +81,24 @@ __host__ __device__ inline void fill_consts(StepArgs& a) {
                                   phi1d(0, a.urx), phi1d(1, a.urx), phi1d(-1, a.urx),
                                   phi1d(0, a.ury), phi1d(1, a.ury), phi1d(-1, a.ury),
                                   a.urx * a.urx + 1.0 / 3.0, a.ury * a.ury + 1.0 / 3.0,
-                                  (c4 - kap) / 3.0, c4 - kap * kap, kap, a.kread == 0 ? -1.0 : 0.0};
+                                  (c4 - kap) / 3.0, c4 - kap * kap, kap, a.kread == 0 ? -1.0 : 0.0,
+                                  -a.rho0, a.w_nu - a.w3, 2.0 * (a.w3 - a.w4), a.w_nu - 2.0 * a.w3 + a.w4,
+                                  (a.w_nu - a.w4) / 3.0, a.w3 - 1.0, a.w4 - 1.0, (a.w_nu - 1.0) / 3.0,
+                                  -(c4 - kap * kap), -a.w_nu, -a.w3, -a.w4};
     for (int k = 0; k < kNumConsts; ++k) {
         a.cd[k] = v[k];
         a.cf[k] = (float)v[k];
     }
+    // in FP32 the combinations are those of the rounded rates
+    const float w = a.cf[0], w3 = a.cf[1], w4 = a.cf[2];
+    a.cf[19] = w - w3;
+    a.cf[20] = 2.0f * (w3 - w4);
+    const float w2 = w - 2.0f * w3;
+    a.cf[21] = w2 + w4;
+    const float d = w - w4;
+    a.cf[22] = (float)(1.0 / 3.0) * d;
+    a.cf[23] = w3 - 1.0f;
+    a.cf[24] = w4 - 1.0f;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -172,42 +189,132 @@ __device__ __forceinline__ void vstore(S* p, const typename Conv<S>::T (&v)[VEC]
     *reinterpret_cast<R*>(p) = r;
 }
 
+// ---------------------------------------------------------------------------------------
+// Arithmetic of the collision, written with explicit fused multiply-adds: every kernel family
+// then rounds alike, whatever the compiler would contract in its own context, and a pair of
+// FP32 nodes can be collided by Blackwell's two-wide FP32 instructions (F2: one instruction for
+// both nodes; each half rounds as the scalar instruction does).  The two-wide instructions have
+// the FLOP rate of the scalar ones (measured 73.6 against 73.7 TFLOP/s) from half the issue slots.
+struct F2 {
+    unsigned long long v;
+};
+template <typename P> struct PairOf {
+    static constexpr bool value = false;
+};
+template <> struct PairOf<F2> {
+    static constexpr bool value = true;
+};
+__device__ __forceinline__ F2 f2_make(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_split(F2 a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ float f2_lo(F2 a) {
+    float lo, hi;
+    f2_split(a, lo, hi);
+    return lo;
+}
+__device__ __forceinline__ float f2_hi(F2 a) {
+    float lo, hi;
+    f2_split(a, lo, hi);
+    return hi;
+}
+
+// a literal in the type one instruction works on
+template <typename P> __device__ __forceinline__ P lit(double c) { return P(c); }
+template <> __device__ __forceinline__ F2 lit<F2>(double c) { return f2_make((float)c, (float)c); }
+
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma3(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double fma3(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ F2 fma3(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+// a - b: there is no two-wide subtraction; a + (-1) b rounds the same (adding the negated halves
+// instead lets the assembler fuse a product into the sum, which does not)
+__device__ __forceinline__ F2 sub(F2 a, F2 b) { return fma3(b, f2_make(-1.0f, -1.0f), a); }
+
 // 1/x.  FP32: the hardware approximation (rcp.approx) refined by one Newton-Raphson step,
 // r' = r + r (1 - x r), two FMAs; within an ulp of the rounded quotient and free of any
 // data-dependent branch, so a lattice that has blown up (non-finite populations) steps as fast
 // as a healthy one.  FP64: the correctly rounded reciprocal intrinsic.
-__device__ __forceinline__ float recip(float x) {
+__device__ __forceinline__ float rcp_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float recip(float x) {
+    const float r = rcp_approx(x);
     return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
 __device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
+// 1/x from x and -x, bit for bit recip(x) in both halves
+__device__ __forceinline__ float recip2(float x, float nx) {
+    const float r = rcp_approx(x);
+    return __fmaf_rn(r, __fmaf_rn(nx, r, 1.0f), r);
+}
+__device__ __forceinline__ F2 recip2(F2 x, F2 nx) {
+    const F2 r = f2_make(rcp_approx(f2_lo(x)), rcp_approx(f2_hi(x)));
+    return fma3(r, fma3(nx, r, f2_make(1.0f, 1.0f)), r);
+}
 
-// Per-launch constants of the collision in the collision precision.
+// Per-launch constants of the collision in the type it works on (the entries of the constant
+// table; see kNumConsts).
 template <typename T> struct Consts {
     T w, w3, w4, rho0, urx, ury;
-    T Px[3], Py[3];      // phi_s(u_ref) for s = 0, +1, -1 (shift factors)
-    T Xr, Yr;            // mu_2(u_ref) = u_ref^2 + c_s^2 per axis
-    T ka, kb;            // cumulant coefficients (see kNumConsts)
+    T Xr, Yr;                // mu_2(u_ref) = u_ref^2 + c_s^2 per axis
+    T ka, kb, nkb;           // cumulant coefficients
+    T nrho0;                 // -rho0
+    T ww3, rr, qq;           // w - w3, 2 (w3 - w4), w - 2 w3 + w4
+    T sw4;                   // c_s^2 (w - w4)
+    T nc3, nc4, sw1;         // w3 - 1, w4 - 1, c_s^2 (w - 1)
+    T nw, nw3, nw4;          // -w, -w3, -w4
 };
 template <typename T> __device__ __forceinline__ const T* const_table(const StepArgs& a);
 template <> __device__ __forceinline__ const float* const_table<float>(const StepArgs& a) { return a.cf; }
 template <> __device__ __forceinline__ const double* const_table<double>(const StepArgs& a) { return a.cd; }
 
 template <typename T>
-__device__ __forceinline__ Consts<T> make_consts(const StepArgs& a) {
-    const T* t = const_table<T>(a);
+__device__ __forceinline__ Consts<T> make_consts_table(const T* t) {
     Consts<T> c;
     c.w = t[0]; c.w3 = t[1]; c.w4 = t[2]; c.rho0 = t[3]; c.urx = t[4]; c.ury = t[5];
-    c.Px[0] = t[6]; c.Px[1] = t[7]; c.Px[2] = t[8];
-    c.Py[0] = t[9]; c.Py[1] = t[10]; c.Py[2] = t[11];
     c.Xr = t[12]; c.Yr = t[13];
-    c.ka = t[14]; c.kb = t[15];
+    c.ka = t[14]; c.kb = t[15]; c.nkb = t[26];
+    c.nrho0 = t[18];
+    c.nw = t[27]; c.nw3 = t[28]; c.nw4 = t[29];
+    c.ww3 = t[19]; c.rr = t[20]; c.qq = t[21];
+    c.sw4 = t[22];
+    c.nc3 = t[23]; c.nc4 = t[24]; c.sw1 = t[25];
     return c;
+}
+template <typename T>
+__device__ __forceinline__ Consts<T> make_consts(const StepArgs& a) {
+    return make_consts_table<T>(const_table<T>(a));
 }
 
 // ---------------------------------------------------------------------------------------
-// Per-node collision (App. B) on shifted populations g_i = f_i - s_i.
+// Per-node collision (App. B) on shifted populations g_i = f_i - s_i.  P is the type one
+// instruction works on: double, float, or F2 (two FP32 nodes).
 //
 // Every model of App. B relaxes the moments of f towards those of f^eq with the same rho
 // and u, through a transform that is linear in f for the node's u, and keeps the conserved
@@ -224,34 +331,304 @@ __device__ __forceinline__ Consts<T> make_consts(const StepArgs& a) {
 // is what makes FP32 arithmetic on FP16-stored populations accurate, and the stored mass and
 // momentum change only by the rounding of D.  rho, ux, uy of the pre-collision state are
 // returned for diagnostics.  SHIFT = false is the default shift s = w rho0 (u_ref = 0), which
-// keeps the shift constants out of the arithmetic.  EQ = 2 (BGK only) uses the second-order
-// equilibrium of Sec. 2 in population space; EQ = 3 (BGK only) the partial third-order one of
-// Fig. 4 (Hermite A^eq_22 = 0: M^eq_22 without its rho u_x^2 u_y^2 term).
-template <int MODEL, int EQ, typename T, bool SHIFT>
-__device__ __forceinline__ void collide(const T (&g)[9], T (&o)[9], const Consts<T>& c, T& rho_out, T& ux_out,
-                                        T& uy_out) {
-    const T cs2 = T(1) / T(3);
-    const T w = c.w, w3 = c.w3, w4 = c.w4;
-    // x-sums of each row of the velocity set (xi_y = +1, 0, -1) with weights 1, xi_x, xi_x^2
+// keeps the shift constants out of the arithmetic.
+//
+// With a21 = 2 ux n11 + uy n20, a12 = 2 uy n11 + ux n02, R = 2 (ux n12 + uy n21) and
+// Q = ux a12 + uy a21 = ux^2 n02 + uy^2 n20 + 4 ux uy n11 the models are
+//   RM, BGK (Eq. RMcoll)       D21 = w3 n21, D12 = w3 n12, D22 = w4 n22;
+//   HM, PR (Hermite moments: A_2 = n_2, A_21 = n_21, A_12 = n_12, A_22 = n_22 - c_s^2 (n_20 + n_02);
+//      Eq. HM2RM_Q9)           D22 = w4 A_22 + c_s^2 (D20 + D02); PR: w3 = w4 = 1;
+//   RR (Eqs. HMColl_Q9, RRformulas_D2Q9: third- and fourth-order A^neq from the recursion, a21, a12
+//      and Q; A* = A^eq + (1 - w) A^neq_rec)
+//                              D21 = n21 - (1 - w3) a21, ..., D22 = A_22 - (1 - w4) Q + c_s^2 (D20 + D02);
+//   CM, CHM, K: central moments k = S(-u) n of f^neq (binomial shift, first-order parts vanish),
+//      relaxed by order (d = rates . k), shifted back D = S(u) d; folded into one expression in n
+//      (k21 = n21 - a21, k12 = n12 - a12, k22 = n22 - R + Q)
+//                              D21 = w3 n21 + (w - w3) a21,   D12 = w3 n12 + (w - w3) a12,
+//                              D22 = w4 n22 + (w3 - w4) R + (w - 2 w3 + w4) Q + (d22 - w4 k22).
+//      CHM: the central Hermite A~_22 = K~_22 - c_s^2 (K~_20 + K~_02) relaxes with w4, the second
+//      order with w (Eqs. CHpoly, CHMcoll): d22 = w4 k22 + c_s^2 (w - w4) (n20 + n02).
+//      K: the cumulant C22 = K22 - (K20 K02 + 2 K11^2)/rho relaxes to 0 and K22* is rebuilt with
+//      second-order central moments kappa n (deviations from the equilibrium central moments
+//      rho c_s^2, 0, rho c_s^4): kappa = 1 - w for the post-collision values (the paper's K), 1 or 0
+//      for the pre-collision / equilibrium readings.  With S = n20 + n02, P = n20 n02 + 2 n11^2 and
+//      c4 = 1 - w4: C22 = k22 - c_s^2 S - P / rho, K22* = c4 C22 + c_s^2 kappa S + kappa^2 P / rho, so
+//      d22 = k22 - K22* = w4 k22 + ka S + kb P / rho, ka = c_s^2 (c4 - kappa), kb = c4 - kappa^2.
+//
+// FP64: the FP64 pipe bounds the kernels, so the expressions share what they can and leave no
+// negation over: j and 1/rho are formed negated, E = M(s) - M^eq enters n by additions.
+// Operations of one node, the reciprocal's aside: BGK 58 .. K 83 (SHIFT 10 more); against the
+// expressions of collide_f32 a step of 128 x 128 BGK takes 11.0 us instead of 13.7, 67 x 37 CHM
+// 16.4 us instead of 18.5.
+template <int MODEL, bool SHIFT>
+__device__ __forceinline__ void collide_f64(const double (&g)[9], double (&o)[9], const Consts<double>& c,
+                                            double& rho_out, double& ux_out, double& uy_out) {
+    using P = double;
+    const P cs2 = P(1.0 / 3.0), ncs2 = P(-1.0 / 3.0);
+    const P w = c.w;
+    // row sums of the velocity set (xi_y = +1, 0, -1): weights 1 (a), xi_x (d), xi_x^2 (s)
+    const P s56 = add(g[5], g[6]), d56 = sub(g[5], g[6]);
+    const P s78 = add(g[8], g[7]), d87 = sub(g[8], g[7]);
+    const P s13 = add(g[1], g[3]), d31 = sub(g[3], g[1]);
+    const P a0p = add(g[2], s56), a0m = add(g[4], s78), a0z = add(g[0], s13);
+    // raw moments of g (App. B, M_pq = sum xi_x^p xi_y^q g); sum s = rho0, sum xi s = rho0 u_ref
+    const P m02 = add(a0p, a0m), njy = sub(a0m, a0p);
+    const P drho = add(m02, a0z);
+    const P m22 = add(s56, s78), m21 = sub(s56, s78);
+    const P m12 = add(d56, d87), m11 = sub(d56, d87);
+    const P m20 = add(s13, m22), njx = sub(d31, m12);
+    const P rho = add(drho, c.rho0);
+    const P nir = -recip(rho);
+    P ux, uy, dx, dy;
+    if (SHIFT) {
+        // u - u_ref = (j - drho u_ref) / rho, j the momentum of g
+        dx = mul(fma3(c.urx, drho, njx), nir);
+        dy = mul(fma3(c.ury, drho, njy), nir);
+        ux = add(dx, c.urx);
+        uy = add(dy, c.ury);
+    } else {
+        ux = mul(njx, nir);
+        uy = mul(njy, nir);
+    }
+    rho_out = rho; ux_out = ux; uy_out = uy;
+
+    // non-equilibrium raw moments n = M(g) + E, E_pq = M_pq(s) - M^eq_pq (Eq. extendedFeq)
+    const P e = mul(ncs2, drho);
+    P n20, n02, n11, n21, n12, n22;
+    if (SHIFT) {
+        // E_20 = -(j_x u_x + rho0 ur_x (u_x - ur_x) + cs2 drho), E_22 = E_20 Y + Xr (E_02 + drho Y)
+        const P qx = mul(dx, c.nrho0), qy = mul(dy, c.nrho0);
+        const P Y = fma3(uy, uy, cs2);
+        const P eX = fma3(njx, ux, fma3(c.urx, qx, e)), eY = fma3(njy, uy, fma3(c.ury, qy, e));
+        n20 = add(m20, eX);
+        n02 = add(m02, eY);
+        n11 = fma3(njx, uy, fma3(c.urx, qy, m11));
+        n21 = fma3(uy, eX, fma3(c.Xr, qy, m21));
+        n12 = fma3(ux, eY, fma3(c.Yr, qx, m12));
+        n22 = fma3(Y, fma3(c.Xr, drho, eX), fma3(c.Xr, eY, m22));
+    } else {
+        // E_20 = -(j_x u_x + cs2 drho), E_21 = -X j_y, E_22 = -(Y j_x u_x + cs2 (j_y u_y + cs2 drho))
+        const P X = fma3(ux, ux, cs2), Y = fma3(uy, uy, cs2);
+        const P pX = mul(njx, ux), eY = fma3(njy, uy, e);
+        n20 = add(m20, add(pX, e));
+        n02 = add(m02, eY);
+        n11 = fma3(njx, uy, m11);
+        n21 = fma3(X, njy, m21);
+        n12 = fma3(Y, njx, m12);
+        n22 = fma3(Y, pX, fma3(cs2, eY, m22));
+    }
+    // D = n - n* (the moments the collision removes), per model; BGK's one rate is left to the
+    // coefficients of the back-transform (D = n there)
+    P D20 = n20, D02 = n02, D11 = n11, D21 = n21, D12 = n12, D22 = n22;
+    if (MODEL != BGK) {
+        D20 = mul(w, n20); D02 = mul(w, n02); D11 = mul(w, n11);
+    }
+    if (MODEL == BGK) {
+    } else if (MODEL == RM) {
+        // Eq. RMcoll
+        D21 = mul(c.w3, n21); D12 = mul(c.w3, n12); D22 = mul(c.w4, n22);
+    } else if (MODEL == HM) {
+        // Hermite moments: A_2 = n_2, A_21 = n_21, A_12 = n_12 (conserved parts vanish),
+        // A_22 = n_22 - c_s^2 (n_20 + n_02); relaxed, back with Eq. HM2RM_Q9:
+        // D22 = w4 A_22 + c_s^2 (D20 + D02)
+        D21 = mul(c.w3, n21); D12 = mul(c.w3, n12);
+        D22 = fma3(c.sw4, add(n20, n02), mul(c.w4, n22));
+    } else if (MODEL == PR) {
+        // HM with omega3 = omega4 = 1
+        D22 = fma3(c.sw1, add(n20, n02), n22);
+    } else {
+        // a21 = 2 ux n11 + uy n20, a12 = 2 uy n11 + ux n02 and
+        // Q = ux a12 + uy a21 = ux^2 n02 + uy^2 n20 + 4 ux uy n11
+        const P t = add(n11, n11);
+        const P a21 = fma3(ux, t, mul(uy, n20)), a12 = fma3(uy, t, mul(ux, n02));
+        const P Q = fma3(ux, a12, mul(uy, a21));
+        if (MODEL == RR) {
+            // Eqs. HMColl_Q9, RRformulas_D2Q9: third/fourth-order A^neq from the recursion
+            // (a21, a12, Q), A* = A^eq + (1 - omega) A^neq_rec, so D = A^neq - (1 - omega) A^neq_rec
+            D21 = fma3(c.nc3, a21, n21);
+            D12 = fma3(c.nc3, a12, n12);
+            D22 = fma3(c.sw1, add(n20, n02), fma3(c.nc4, Q, n22));
+        } else {
+            // central moments k = S(-u) n of f^neq (binomial shift, first-order parts vanish),
+            // relaxed by order (d = rates . k), shifted back D = S(u) d.  The three linear steps
+            // are folded into one expression in n: with R = 2 (ux n12 + uy n21) one has
+            // k21 = n21 - a21, k12 = n12 - a12, k22 = n22 - R + Q, and
+            //   D21 = w3 n21 + (w - w3) a21,   D12 = w3 n12 + (w - w3) a12,
+            //   D22 = w4 n22 + (w3 - w4) R + (w - 2 w3 + w4) Q + (model terms),
+            // the model terms being d22 - w4 k22 (zero for CM).
+            D21 = fma3(c.ww3, a21, mul(c.w3, n21));
+            D12 = fma3(c.ww3, a12, mul(c.w3, n12));
+            const P R = fma3(ux, n12, mul(uy, n21));
+            D22 = fma3(c.qq, Q, fma3(c.rr, R, mul(c.w4, n22)));
+            if (MODEL == CHM) {
+                // central Hermite: A~_22 = K~_22 - c_s^2 (K~_20 + K~_02) relaxed with w4, the
+                // second order with w (Eqs. CHpoly, CHMcoll): d22 = w4 A~_22 + c_s^2 (d20 + d02)
+                // = w4 k22 + c_s^2 (w - w4) (n20 + n02)
+                D22 = fma3(c.sw4, add(n20, n02), D22);
+            } else if (MODEL != CM) {
+                // cumulants: C22 = K22 - (K20 K02 + 2 K11^2)/rho relaxes to 0 and K22* is rebuilt
+                // with second-order central moments kappa n (written for deviations from the
+                // equilibrium central moments rho c_s^2, 0, rho c_s^4): kappa = 1 - w for the
+                // post-collision values (the paper's K), 1 or 0 for the pre-collision / equilibrium
+                // readings.  With S = n20 + n02, P = n20 n02 + 2 n11^2 and c4 = 1 - w4:
+                // C22 = k22 - c_s^2 S - P / rho, K22* = c4 C22 + c_s^2 kappa S + kappa^2 P / rho, so
+                // d22 = k22 - K22* = w4 k22 + ka S + kb P / rho with the per-launch constants
+                // ka = c_s^2 (c4 - kappa), kb = c4 - kappa^2
+                const P PP = fma3(n20, n02, mul(t, n11));
+                D22 = fma3(mul(c.nkb, nir), PP, fma3(c.ka, add(n20, n02), D22));
+            }
+        }
+    }
+
+    // g* = g - (Eq. Q9postCollVDF_RM applied to D, with D_00 = D_10 = D_01 = 0)
+    const P nh = MODEL == BGK ? mul(P(-0.5), w) : P(-0.5);
+    const P nq = MODEL == BGK ? mul(P(-0.25), w) : P(-0.25);
+    const P A = sub(D20, D22), B = sub(D02, D22);
+    o[0] = MODEL == BGK ? fma3(w, add(A, D02), g[0]) : add(g[0], add(A, D02));
+    o[1] = fma3(nh, sub(A, D12), g[1]);
+    o[3] = fma3(nh, add(A, D12), g[3]);
+    o[2] = fma3(nh, sub(B, D21), g[2]);
+    o[4] = fma3(nh, add(B, D21), g[4]);
+    const P E = add(D22, D11), F = sub(D22, D11), U = add(D21, D12), V = sub(D21, D12);
+    o[5] = fma3(nq, add(E, U), g[5]);
+    o[7] = fma3(nq, sub(E, U), g[7]);
+    o[6] = fma3(nq, add(F, V), g[6]);
+    o[8] = fma3(nq, sub(F, V), g[8]);
+}
+
+
+// FP32 (one node: float, two: F2).  The operations, their order and what is fused are fixed here,
+// so that every kernel form and both widths give the same bits; 16-bit storage needs that most: one
+// population rounded the other way spreads until, after some hundred steps, two BF16 runs differ by
+// as much as either does from FP64.  Products that a sum takes up fused are not formed again.
+// Operations of one node: BGK 80, K 103 (the expressions of collide_f64 would be 60 and 85 and the
+// time-fused kernel 8-11 % faster, 1042 us against 1157 a step of 16384^2 K; they round differently).
+template <int MODEL, typename P, bool SHIFT>
+__device__ __forceinline__ void collide_f32(const P (&g)[9], P (&o)[9], const Consts<P>& c, P& rho_out, P& ux_out,
+                                            P& uy_out) {
+    constexpr bool ONE_BY_ONE = MODEL == BGK || MODEL == RM || MODEL == HM;   // D21 = w3 n21, D12 = w3 n12
+    const P cs2 = lit<P>(1.0 / 3.0), ncs2 = lit<P>(-1.0 / 3.0);
+    const P w = c.w, nw = c.nw;
+    const P w3 = MODEL == BGK ? c.w : c.w3, nw3 = MODEL == BGK ? c.nw : c.nw3;
+    const P w4 = MODEL == BGK ? c.w : c.w4, nw4 = MODEL == BGK ? c.nw : c.nw4;
+    const P a0p = add(add(g[6], g[2]), g[5]), a1p = sub(g[5], g[6]), a2p = add(g[5], g[6]);
+    const P a0z = add(add(g[3], g[0]), g[1]), a1z = sub(g[1], g[3]), a2z = add(g[1], g[3]);
+    const P a0m = add(add(g[7], g[4]), g[8]), a1m = sub(g[8], g[7]), a2m = add(g[8], g[7]);
+    const P drho = add(add(a0p, a0z), a0m);
+    P jx = add(add(a1p, a1z), a1m), jy = sub(a0p, a0m);
+    const P m20 = add(add(a2p, a2z), a2m), m02 = add(a0p, a0m), m11 = sub(a1p, a1m);
+    const P m21 = sub(a2p, a2m), m12 = add(a1p, a1m), m22 = add(a2p, a2m);
+    const P rho = add(drho, c.rho0), nrho = sub(c.nrho0, drho);
+    if (SHIFT) {
+        jx = fma3(c.rho0, c.urx, jx);
+        jy = fma3(c.rho0, c.ury, jy);
+    }
+    const P irho = recip2(rho, nrho);
+    const P ux = mul(jx, irho), uy = mul(jy, irho);
+    const P uxx = mul(ux, ux), uyy = mul(uy, uy), uxy = mul(ux, uy);
+    rho_out = rho; ux_out = ux; uy_out = uy;
+
+    P n20, n02, n11, n21, n12, n22;
+    if (SHIFT) {
+        constexpr bool SQUARES = MODEL == RR || MODEL == CM || MODEL == CHM || MODEL == CUM;   // uxx, uyy serve twice
+        const P X = SQUARES ? add(uxx, cs2) : fma3(ux, ux, cs2), Y = SQUARES ? add(uyy, cs2) : fma3(uy, uy, cs2);
+        const P dx = sub(ux, c.urx), dy = sub(uy, c.ury);
+        const P dX = mul(dx, add(ux, c.urx)), dY = mul(dy, add(uy, c.ury));
+        n20 = sub(m20, fma3(drho, X, mul(c.rho0, dX)));
+        n02 = sub(m02, fma3(drho, Y, mul(c.rho0, dY)));
+        n11 = sub(m11, fma3(drho, uxy, mul(c.rho0, fma3(dx, uy, mul(c.urx, dy)))));
+        n21 = sub(m21, fma3(drho, mul(X, uy), mul(c.rho0, fma3(c.Xr, dy, mul(dX, uy)))));
+        n12 = sub(m12, fma3(drho, mul(ux, Y), mul(c.rho0, fma3(dx, Y, mul(c.urx, dY)))));
+        n22 = sub(m22, fma3(drho, mul(X, Y), mul(c.rho0, fma3(dX, Y, mul(c.Xr, dY)))));
+    } else {
+        const P X = add(uxx, cs2), Y = add(uyy, cs2);
+        n20 = sub(m20, fma3(cs2, drho, mul(rho, uxx)));
+        n02 = sub(m02, fma3(cs2, drho, mul(rho, uyy)));
+        n11 = fma3(nrho, uxy, m11);
+        n21 = fma3(mul(nrho, X), uy, m21);
+        n12 = fma3(mul(nrho, ux), Y, m12);
+        n22 = sub(m22, fma3(drho, mul(X, Y), mul(c.rho0, fma3(cs2, uyy, mul(uxx, Y)))));
+    }
+
+    const P D02 = mul(w, n02), DS = fma3(w, n20, D02);   // DS = D20 + D02
+    P D21, D12, D22;
+    if (MODEL == BGK || MODEL == RM) {
+        D21 = mul(w3, n21); D22 = mul(w4, n22);
+    } else if (MODEL == HM || MODEL == PR) {
+        const P a22 = fma3(ncs2, add(n20, n02), n22);
+        if (MODEL == HM) {
+            D21 = mul(w3, n21);
+            D22 = fma3(cs2, DS, mul(w4, a22));
+        } else {
+            D21 = n21; D12 = n12;
+            D22 = fma3(cs2, DS, a22);
+        }
+    } else {
+        const P t = add(n11, n11);
+        const P a21 = SHIFT ? fma3(uy, n20, mul(ux, t)) : fma3(ux, t, mul(uy, n20));
+        const P a12 = SHIFT ? fma3(ux, n02, mul(uy, t)) : fma3(uy, t, mul(ux, n02));
+        if (MODEL == RR) {
+            const P a22 = fma3(uxy, add(t, t), fma3(uyy, n20, mul(uxx, n02)));
+            D21 = fma3(c.nc3, a21, n21);
+            D12 = fma3(c.nc3, a12, n12);
+            D22 = fma3(cs2, DS, fma3(c.nc4, a22, fma3(ncs2, add(n20, n02), n22)));
+        } else {
+            const P R = fma3(ux, n12, mul(uy, n21));
+            const P Q = fma3(uxy, add(t, t), fma3(uxx, n02, mul(uyy, n20)));
+            D21 = fma3(w3, n21, mul(c.ww3, a21));
+            D12 = fma3(w3, n12, mul(c.ww3, a12));
+            D22 = fma3(c.qq, Q, fma3(w4, n22, mul(c.rr, R)));
+            if (MODEL == CHM) {
+                D22 = fma3(c.sw4, add(n20, n02), D22);
+            } else if (MODEL != CM) {
+                const P PP = fma3(n20, n02, mul(t, n11));
+                D22 = add(D22, fma3(c.ka, add(n20, n02), mul(mul(c.kb, irho), PP)));
+            }
+        }
+    }
+
+    const P h = lit<P>(0.5), nh = lit<P>(-0.5), nq = lit<P>(-0.25);
+    const P nA = fma3(nw, n20, D22), B = sub(D02, D22);   // -(D20 - D22), D02 - D22
+    o[0] = add(g[0], (MODEL == BGK || MODEL == RM) ? fma3(nw4, n22, DS) : sub(DS, D22));
+    P U, V;   // D21 + D12, D21 - D12
+    if (ONE_BY_ONE) {
+        o[1] = fma3(h, fma3(w3, n12, nA), g[1]);
+        o[3] = fma3(h, fma3(nw3, n12, nA), g[3]);
+        o[2] = fma3(nh, fma3(nw3, n21, B), g[2]);
+        o[4] = fma3(nh, fma3(w3, n21, B), g[4]);
+        U = fma3(w3, n12, D21);
+        V = fma3(nw3, n12, D21);
+    } else {
+        o[1] = fma3(h, add(nA, D12), g[1]);
+        o[3] = fma3(h, sub(nA, D12), g[3]);
+        o[2] = fma3(nh, sub(B, D21), g[2]);
+        o[4] = fma3(nh, add(B, D21), g[4]);
+        U = add(D12, D21);
+        V = sub(D21, D12);
+    }
+    const P E = fma3(w, n11, D22), F = fma3(nw, n11, D22);   // D22 +- D11
+    o[5] = fma3(nq, add(E, U), g[5]);
+    o[7] = fma3(nq, sub(E, U), g[7]);
+    o[6] = fma3(nq, add(F, V), g[6]);
+    o[8] = fma3(nq, sub(F, V), g[8]);
+}
+
+// BGK with the second-order equilibrium of Sec. 2 (EQ = 2, population space) or the partial
+// third-order one of Fig. 4 (EQ = 3: Hermite A^eq_22 = 0, M^eq_22 without its rho u_x^2 u_y^2 term),
+// u_ref = 0.
+template <int EQ, typename T>
+__device__ __forceinline__ void collide_truncated(const T (&g)[9], T (&o)[9], const Consts<T>& c, T& rho_out,
+                                                  T& ux_out, T& uy_out) {
+    const T cs2 = T(1) / T(3), w = c.w;
     const T a0p = (g[6] + g[2]) + g[5], a1p = g[5] - g[6], a2p = g[5] + g[6];
     const T a0z = (g[3] + g[0]) + g[1], a1z = g[1] - g[3], a2z = g[1] + g[3];
     const T a0m = (g[7] + g[4]) + g[8], a1m = g[8] - g[7], a2m = g[8] + g[7];
-    // raw moments of g (App. B, M_pq = sum xi_x^p xi_y^q g); sum s = rho0, sum xi s = rho0 u_ref
-    const T drho = (a0p + a0z) + a0m;
-    T jx = (a1p + a1z) + a1m;
-    T jy = a0p - a0m;
-    const T m20 = (a2p + a2z) + a2m, m02 = a0p + a0m, m11 = a1p - a1m;
-    const T m21 = a2p - a2m, m12 = a1p + a1m, m22 = a2p + a2m;
-    const T rho = c.rho0 + drho;
-    if (SHIFT) {
-        jx += c.rho0 * c.urx;
-        jy += c.rho0 * c.ury;
-    }
+    const T drho = (a0p + a0z) + a0m, rho = c.rho0 + drho;
+    const T jx = (a1p + a1z) + a1m, jy = a0p - a0m;
     const T irho = recip(rho);
     const T ux = jx * irho, uy = jy * irho;
     const T uxx = ux * ux, uyy = uy * uy;
     rho_out = rho; ux_out = ux; uy_out = uy;
-
     if (EQ == 2) {
         // second-order equilibrium (Sec. 2, Hermite reading), shift s = w rho0 (u_ref = 0):
         // f^eq_i = w_i rho (1 + 3 xi.u + 4.5 (xi.u)^2 - 1.5 u^2); BGK in population space
@@ -278,98 +655,17 @@ __device__ __forceinline__ void collide(const T (&g)[9], T (&o)[9], const Consts
         for (int i = 0; i < 9; ++i) o[i] = geq[i] + cc * fn[i];
         return;
     }
-
-    // non-equilibrium raw moments n = M(g) - (M^eq(rho, u) - M(s)) (Eq. extendedFeq)
-    T n20, n02, n11, n21, n12, n22;
-    if (SHIFT) {
-        const T X = uxx + cs2, Y = uyy + cs2;                   // mu_2(u_x), mu_2(u_y)
-        const T dx = ux - c.urx, dy = uy - c.ury;               // mu_1(u) - mu_1(u_ref)
-        const T dX = dx * (ux + c.urx), dY = dy * (uy + c.ury); // mu_2(u) - mu_2(u_ref)
-        const T r0 = c.rho0;
-        n20 = m20 - (drho * X + r0 * dX);
-        n02 = m02 - (drho * Y + r0 * dY);
-        n11 = m11 - (drho * (ux * uy) + r0 * (dx * uy + c.urx * dy));
-        n21 = m21 - (drho * (X * uy) + r0 * (dX * uy + c.Xr * dy));
-        n12 = m12 - (drho * (ux * Y) + r0 * (dx * Y + c.urx * dY));
-        n22 = m22 - (drho * (X * Y) + r0 * (dX * Y + c.Xr * dY));
-    } else {
-        const T Y = uyy + cs2;
-        const T rX = rho * (uxx + cs2);
-        n20 = m20 - (cs2 * drho + rho * uxx);
-        n02 = m02 - (cs2 * drho + rho * uyy);
-        n11 = m11 - rho * (ux * uy);
-        n21 = m21 - rX * uy;
-        n12 = m12 - (rho * ux) * Y;
-        n22 = m22 - (drho * ((uxx + cs2) * Y) + c.rho0 * (uxx * Y + cs2 * uyy));
-    }
-    if (EQ == 3) n22 += rho * (uxx * uyy);   // M^eq_22 of the partial third-order equilibrium
-
-    // D = n - n* (the moments the collision removes), per model
-    T D20, D02, D11, D21, D12, D22;
-    if (MODEL == BGK || MODEL == RM) {
-        // Eq. RMcoll (BGK: one rate for every order)
-        const T r3 = (MODEL == BGK) ? w : w3, r4 = (MODEL == BGK) ? w : w4;
-        D20 = w * n20; D02 = w * n02; D11 = w * n11;
-        D21 = r3 * n21; D12 = r3 * n12; D22 = r4 * n22;
-    } else if (MODEL == HM || MODEL == PR) {
-        // Hermite moments: A_2 = n_2, A_21 = n_21, A_12 = n_12 (conserved parts vanish),
-        // A_22 = n_22 - c_s^2 (n_20 + n_02); relaxed, back with Eq. HM2RM_Q9
-        D20 = w * n20; D02 = w * n02; D11 = w * n11;
-        if (MODEL == HM) {
-            D21 = w3 * n21; D12 = w3 * n12;
-            D22 = w4 * (n22 - cs2 * (n20 + n02)) + cs2 * (D20 + D02);
-        } else {   // PR: omega3 = omega4 = 1
-            D21 = n21; D12 = n12;
-            D22 = (n22 - cs2 * (n20 + n02)) + cs2 * (D20 + D02);
-        }
-    } else if (MODEL == RR) {
-        // Eqs. HMColl_Q9, RRformulas_D2Q9: third/fourth-order A^neq from the recursion,
-        // A* = A^eq + (1 - omega) A^neq_rec, so D = A^neq - (1 - omega) A^neq_rec
-        const T a21 = uy * n20 + T(2) * ux * n11;
-        const T a12 = ux * n02 + T(2) * uy * n11;
-        const T a22 = uyy * n20 + uxx * n02 + T(4) * ux * uy * n11;
-        const T c3 = T(1) - w3, c4 = T(1) - w4;
-        D20 = w * n20; D02 = w * n02; D11 = w * n11;
-        D21 = n21 - c3 * a21; D12 = n12 - c3 * a12;
-        D22 = (n22 - cs2 * (n20 + n02)) - c4 * a22 + cs2 * (D20 + D02);
-    } else {
-        // central moments k = S(-u) n of f^neq (binomial shift, first-order parts vanish),
-        // relaxed by order (d = rates . k), shifted back D = S(u) d.  The three linear steps are
-        // folded into one expression in n: with a21 = 2 ux n11 + uy n20, a12 = 2 uy n11 + ux n02,
-        // R = 2 (ux n12 + uy n21) and Q = ux^2 n02 + uy^2 n20 + 4 ux uy n11 one has
-        // k21 = n21 - a21, k12 = n12 - a12, k22 = n22 - R + Q, and
-        //   D21 = w3 n21 + (w - w3) a21,   D12 = w3 n12 + (w - w3) a12,
-        //   D22 = w4 n22 + (w3 - w4) R + (w - 2 w3 + w4) Q + (model terms),
-        // the model terms being d22 - w4 k22 (zero for CM).
-        const T uxy = ux * uy;
-        const T a21 = T(2) * ux * n11 + uy * n20, a12 = T(2) * uy * n11 + ux * n02;
-        const T R = T(2) * (ux * n12 + uy * n21);
-        const T Q = uxx * n02 + uyy * n20 + T(4) * uxy * n11;
-        D20 = w * n20; D02 = w * n02; D11 = w * n11;
-        D21 = w3 * n21 + (w - w3) * a21;
-        D12 = w3 * n12 + (w - w3) * a12;
-        T D22c = w4 * n22 + (w3 - w4) * R + (w - T(2) * w3 + w4) * Q;
-        if (MODEL == CHM) {
-            // central Hermite: A~_22 = K~_22 - c_s^2 (K~_20 + K~_02) relaxed with w4, the
-            // second order with w (Eqs. CHpoly, CHMcoll): d22 = w4 A~_22 + c_s^2 (d20 + d02)
-            // = w4 k22 + c_s^2 (w - w4) (n20 + n02)
-            D22c += (cs2 * (w - w4)) * (n20 + n02);
-        } else if (MODEL != CM) {
-            // cumulants: C22 = K22 - (K20 K02 + 2 K11^2)/rho relaxes to 0 and K22* is rebuilt
-            // with second-order central moments kappa n (written for deviations from the
-            // equilibrium central moments rho c_s^2, 0, rho c_s^4): kappa = 1 - w for the
-            // post-collision values (the paper's K), 1 or 0 for the pre-collision / equilibrium
-            // readings.  With S = n20 + n02, P = n20 n02 + 2 n11^2 and c4 = 1 - w4:
-            // C22 = k22 - c_s^2 S - P / rho, K22* = c4 C22 + c_s^2 kappa S + kappa^2 P / rho, so
-            // d22 = k22 - K22* = w4 k22 + ka S + kb P / rho with the per-launch constants
-            // ka = c_s^2 (c4 - kappa), kb = c4 - kappa^2
-            const T P = n20 * n02 + T(2) * n11 * n11;
-            D22c += c.ka * (n20 + n02) + (c.kb * irho) * P;
-        }
-        D22 = D22c;
-    }
-
-    // g* = g - (Eq. Q9postCollVDF_RM applied to D, with D_00 = D_10 = D_01 = 0)
+    const T m20 = (a2p + a2z) + a2m, m02 = a0p + a0m, m11 = a1p - a1m;
+    const T m21 = a2p - a2m, m12 = a1p + a1m, m22 = a2p + a2m;
+    const T Y = uyy + cs2;
+    const T rX = rho * (uxx + cs2);
+    const T n20 = m20 - (cs2 * drho + rho * uxx);
+    const T n02 = m02 - (cs2 * drho + rho * uyy);
+    const T n11 = m11 - rho * (ux * uy);
+    const T n21 = m21 - rX * uy;
+    const T n12 = m12 - (rho * ux) * Y;
+    const T n22 = m22 - (drho * ((uxx + cs2) * Y) + c.rho0 * (uxx * Y + cs2 * uyy)) + rho * (uxx * uyy);
+    const T D20 = w * n20, D02 = w * n02, D11 = w * n11, D21 = w * n21, D12 = w * n12, D22 = w * n22;
     const T h = T(0.5), q = T(0.25);
     o[0] = g[0] - (D22 - (D20 + D02));
     o[1] = g[1] - h * ((D20 - D22) - D12);
@@ -380,6 +676,13 @@ __device__ __forceinline__ void collide(const T (&g)[9], T (&o)[9], const Consts
     o[6] = g[6] - q * ((D22 - D11) + (D21 - D12));
     o[7] = g[7] - q * ((D22 + D11) - (D12 + D21));
     o[8] = g[8] - q * ((D22 - D11) + (D12 - D21));
+}
+
+template <int MODEL, int EQ, typename P, bool SHIFT>
+__device__ __forceinline__ void collide(const P (&g)[9], P (&o)[9], const Consts<P>& c, P& rho, P& ux, P& uy) {
+    if constexpr (EQ != 4) collide_truncated<EQ, P>(g, o, c, rho, ux, uy);
+    else if constexpr (sizeof(P) == 8 && !PairOf<P>::value) collide_f64<MODEL, SHIFT>(g, o, c, rho, ux, uy);
+    else collide_f32<MODEL, P, SHIFT>(g, o, c, rho, ux, uy);
 }
 
 // Per-thread FP64 accumulators of the blow-up diagnostics (used by the batched sweep).

@@ -34,6 +34,12 @@ bool tile_kernel_f32(bool shifted, int stages, int form, TileKernelInfo* out);
 bool tile_kernel_f16(bool shifted, int stages, int form, TileKernelInfo* out);
 bool tile_kernel_bf16(bool shifted, int stages, int form, TileKernelInfo* out);
 
+// Time-fused step kernel (march_kernel<S, shifted, pairs, roll>, one MarchArgs parameter) per
+// storage; pairs: every lattice of the launch has an even nx; roll: the form for mixed models.
+const void* march_kernel_f32(bool shifted, bool pairs, bool roll);
+const void* march_kernel_f16(bool shifted, bool pairs, bool roll);
+const void* march_kernel_bf16(bool shifted, bool pairs, bool roll);
+
 // Batched persistent sweep kernel for (vector width, CTA size); nullptr if not instantiated.
 const void* batch_kernel_f64(int vec, int block);
 const void* batch_kernel_f32(int vec, int block);
@@ -109,8 +115,8 @@ struct AdjArgs {
     long long plane;
     double w_nu, w3, w4, rho0;
     double urx, ury;     // storage shift velocity
-    double cd[18];       // collision constants as in StepArgs (fill_consts), FP64 and FP32
-    float cf[18];
+    double cd[30];       // collision constants as in StepArgs (fill_consts), FP64 and FP32
+    float cf[30];
 };
 struct AdjointPlan {
     int storage;            // LBM_F64 or LBM_F32 (lambda kept in the collision precision)

@@ -1,0 +1,14 @@
+// Time-fused step kernels for float population storage.
+#include "lbm_march.cuh"
+#include "lbm_internal.h"
+
+namespace lbm {
+template <bool SHIFT, bool PAIRS>
+static const void* march_table(bool roll) {
+    return roll ? (const void*)march_kernel<float, SHIFT, PAIRS, true> : (const void*)march_kernel<float, SHIFT, PAIRS, false>;
+}
+const void* march_kernel_f32(bool shifted, bool pairs, bool roll) {
+    if (pairs) return shifted ? march_table<true, true>(roll) : march_table<false, true>(roll);
+    return shifted ? march_table<true, false>(roll) : march_table<false, false>(roll);
+}
+}  // namespace lbm
