@@ -9,6 +9,7 @@
 #include "lbm.h"
 
 #include "lbm_device.cuh"
+#include "lbm_equilibrium.cuh"
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -34,30 +35,39 @@ __device__ __forceinline__ long long src_offset(int i, int x, int y, const Field
     return (long long)i * a.plane + (long long)ys * a.pitch + xs;
 }
 
+// Measured, 16384^2: FP32 36.6 -> 5.3 ms, FP16 36.6 -> 5.5 ms; 1024^2 FP32 178 -> 47 us (what
+// bounds it is issue: some 500 FP32 and integer instructions a node).
 template <typename S>
-__global__ void init_eq_kernel(S* buf, FieldArgs a, int eq_order, const double* __restrict__ rho,
-                               const double* __restrict__ ux, const double* __restrict__ uy) {
+__global__ void __launch_bounds__(kBlock) init_eq_kernel(S* buf, FieldArgs a, EquilibriumConsts c,
+                                                         const double* __restrict__ rho, const double* __restrict__ ux,
+                                                         const double* __restrict__ uy) {
+    const unsigned n = (unsigned)a.nx * (unsigned)a.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int y = (int)(k / (unsigned)a.nx), x = (int)(k - (unsigned)y * (unsigned)a.nx);
+        S g[9];
+        equilibrium_node<S>(rho[k], ux[k], uy[k], a.rho0, a.urx, a.ury, c, g);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) buf[src_offset(i, x, y, a)] = g[i];
+    }
+}
+
+// The truncated equilibria of BGK (eq_order 2 and 3, u_ref = 0).
+template <typename S>
+__global__ void init_eq_truncated_kernel(S* buf, FieldArgs a, int eq_order, const double* __restrict__ rho,
+                                         const double* __restrict__ ux, const double* __restrict__ uy) {
     const long long n = (long long)a.nx * a.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const int y = (int)(k / a.nx), x = (int)(k - (long long)y * a.nx);
-        const double r = rho[k], vx = ux[k], vy = uy[k];
-        const double dr = r - a.rho0;
+        const double r = rho[k], vx = ux[k], vy = uy[k], dr = r - a.rho0;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const int sx = ex_of(i), sy = ey_of(i);
             double g;
-            if (eq_order >= 3) {
-                // Eq. extendedFeq in product form minus the shift s_i = rho0 P_sx P_sy, with
-                // P_s = phi_s(u_ref) and D_s = phi_s(u) - phi_s(u_ref) written as differences
-                const double Px = phi1d(sx, a.urx), Py = phi1d(sy, a.ury);
-                const double dux = vx - a.urx, sux = vx + a.urx, duy = vy - a.ury, suy = vy + a.ury;
-                const double Dx = sx ? 0.5 * dux * (sux + sx) : -dux * sux;
-                const double Dy = sy ? 0.5 * duy * (suy + sy) : -duy * suy;
-                g = Px * Py * dr + r * (Px * Dy + Dx * (Py + Dy));
-                // partial third order (u_ref = 0): minus rho u_x^2 u_y^2 times the populations
-                // of a unit M_22 (Eq. Q9postCollVDF_RM: 1 at rest, -1/2 on the axes, 1/4 on
-                // the diagonals)
-                if (eq_order == 3) g -= r * (vx * vx) * (vy * vy) * (sx ? -0.5 : 1.0) * (sy ? -0.5 : 1.0);
+            if (eq_order == 3) {
+                // partial third order: minus rho u_x^2 u_y^2 times the populations of a unit M_22
+                // (Eq. Q9postCollVDF_RM: 1 at rest, -1/2 on the axes, 1/4 on the diagonals)
+                g = equilibrium_plain(i, r, vx, vy, a.rho0, a.urx, a.ury);
+                g -= r * (vx * vx) * (vy * vy) * (sx ? -0.5 : 1.0) * (sy ? -0.5 : 1.0);
             } else {
                 const double wi = weight_of(i);
                 const double eu = 3.0 * (sx * vx + sy * vy);
@@ -79,38 +89,179 @@ __global__ void scatter_kernel(S* buf, FieldArgs a, const double* __restrict__ f
     }
 }
 
-template <typename S>
-__global__ void gather_kernel(const S* buf, FieldArgs a, double* f, double* rho, double* ux, double* uy,
-                              double* pxx, double* pxy, double* pyy) {
+// ---- populations and moments out, in FP64 -------------------------------------------------
+// GB300 has 2 FP64 lanes per SM and clock (conversions included) against 128 for FP32: done
+// plainly, rho, u of a node of FP32 populations are 9 conversions, 54 sums and two divisions, and
+// that pipe bounded the kernel (37.4 ms at 16384^2, 16 GB to move).  So FP32 values are widened
+// with integer operations; their sums are taken exactly in FP32 by error-free two-sums (Knuth), two
+// nodes per instruction, and only closed in FP64; u takes one reciprocal for both components by a
+// Newton step from the FP32 one and closes each quotient with its remainder (Markstein).  That
+// leaves 12 FP64 operations a node: 37.4 -> 10.5 ms at 16384^2, 155 -> 55 us at 1024^2; errors as
+// before (rho 1.7e-16, u 1.7e-17 at most, against long double).
+
+// the double of a float's value
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t u = __float_as_uint(v), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)v;   // subnormal, infinite, not a number
+    const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+
+// s + e = a + b exactly
+__device__ __forceinline__ void two_sum(F2 a, F2 b, F2& s, F2& e) {
+    s = add(a, b);
+    const F2 t = sub(s, a);
+    e = add(sub(a, sub(s, t)), sub(b, t));
+}
+// A sum of floats kept as hi + mid + lo: hi and mid hold it exactly unless the terms' exponents
+// differ by more than about 2^20, lo what is below that.
+struct ExactSum {
+    F2 hi, mid, lo;
+    __device__ __forceinline__ explicit ExactSum(F2 x) : hi(x), mid(lit<F2>(0.0)), lo(lit<F2>(0.0)) {}
+    __device__ __forceinline__ void plus(F2 x) {
+        F2 e, e2;
+        two_sum(hi, x, hi, e);
+        two_sum(mid, e, mid, e2);
+        lo = add(lo, e2);
+    }
+    __device__ __forceinline__ void minus(F2 x) { plus(mul(x, lit<F2>(-1.0))); }
+    // the value of one of the two nodes
+    __device__ __forceinline__ double value(int j) const {
+        const float a = j ? f2_hi(hi) : f2_lo(hi), b = j ? f2_hi(mid) : f2_lo(mid), c = j ? f2_hi(lo) : f2_lo(lo);
+        double d = widen(b);
+        if (c != 0.0f) d += widen(c);
+        return widen(a) + d;
+    }
+};
+
+struct MomentOut {
+    double *rho, *ux, *uy, *pxx, *pxy, *pyy;
+    __device__ __forceinline__ bool any() const { return rho || ux || uy || pxx || pxy || pyy; }
+    __device__ __forceinline__ bool second() const { return pxx || pxy || pyy; }
+};
+
+// Moments of one node from its populations, one FP64 sum after another: every storage type's for a
+// node with a non-finite or extreme value, FP64 storage's always (there without the zero terms,
+// which change nothing where the density is finite).
+template <bool ZEROS>
+__device__ __forceinline__ void moments_plain(const double (&g)[9], const FieldArgs& a, const MomentOut& o, long long k) {
+    double dr = 0, jx = 0, jy = 0, sxx = 0, sxy = 0, syy = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int sx = ex_of(i), sy = ey_of(i);
+        dr += g[i];
+        if (ZEROS || sx) jx += sx * g[i];
+        if (ZEROS || sy) jy += sy * g[i];
+        if (ZEROS || sx) sxx += sx * sx * g[i];
+        if (ZEROS || sx * sy) sxy += sx * sy * g[i];
+        if (ZEROS || sy) syy += sy * sy * g[i];
+    }
+    // moments of the shift: sum s = rho0, sum xi s = rho0 u_ref,
+    // sum xi_a xi_b s = rho0 (u_ref,a u_ref,b + c_s^2 delta_ab)
+    const double r = a.rho0 + dr;
+    jx += a.rho0 * a.urx;
+    jy += a.rho0 * a.ury;
+    if (o.rho) o.rho[k] = r;
+    if (o.ux) o.ux[k] = jx / r;
+    if (o.uy) o.uy[k] = jy / r;
+    if (o.pxx) o.pxx[k] = sxx + a.rho0 * (a.urx * a.urx + 1.0 / 3.0);
+    if (o.pxy) o.pxy[k] = sxy + a.rho0 * a.urx * a.ury;
+    if (o.pyy) o.pyy[k] = syy + a.rho0 * (a.ury * a.ury + 1.0 / 3.0);
+}
+
+// FP64 storage: one node per thread.
+__global__ void gather_kernel_f64(const double* buf, FieldArgs a, double* f, MomentOut o) {
     const long long n = (long long)a.nx * a.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const int y = (int)(k / a.nx), x = (int)(k - (long long)y * a.nx);
-        double g[9];
+        double g[9], dr = 0.0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) g[i] = Conv<S>::to_double(buf[src_offset(i, x, y, a)]);
+        for (int i = 0; i < 9; ++i) {
+            g[i] = buf[src_offset(i, x, y, a)];
+            dr += g[i];
+        }
         if (f) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) f[i * n + k] = g[i] + shift_of(i, a.rho0, a.urx, a.ury);
         }
-        if (rho || ux || uy || pxx || pxy || pyy) {
-            double dr = 0, jx = 0, jy = 0, sxx = 0, sxy = 0, syy = 0;
+        if (o.any()) {
+            if (isfinite(dr)) moments_plain<false>(g, a, o, k);
+            else moments_plain<true>(g, a, o, k);
+        }
+    }
+}
+
+// 32- and 16-bit storage: two neighbouring nodes per thread, gathered as in the step kernels.
+// shift: the constants s_i; second: ur_x^2 + c_s^2, rho0 ur_x, ur_y^2 + c_s^2.
+struct GatherConsts {
+    double shift[9], second[3];
+};
+template <typename S>
+__global__ void __launch_bounds__(kBlock) gather_kernel(const S* buf, FieldArgs a, double* f, MomentOut o, GatherConsts c) {
+    const long long n = (long long)a.nx * a.ny;
+    const int lane = threadIdx.x & 31, nseg = (a.nx + 1) / 2;
+    const bool shifted = a.urx != 0.0 || a.ury != 0.0;
+    const unsigned total = (unsigned)a.ny * (unsigned)nseg, stride = gridDim.x * blockDim.x;
+    for (unsigned base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < total; base += stride) {
+        const bool active = base + lane < total;
+        const unsigned s = active ? base + lane : total - 1;
+        const int y = (int)(s / (unsigned)nseg), x0 = 2 * (int)(s - (unsigned)y * (unsigned)nseg);
+        const int nvalid = min(2, a.nx - x0);
+        float g[9][2];
+        gather_pull<S, 2, 1>(buf, a.nx, a.ny, a.pitch, a.plane, y, x0 / 2, nseg, x0, nvalid, lane, g);
+        if (!active) continue;
+        const long long k = (long long)y * a.nx + x0;
+        if (f) {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const int sx = ex_of(i), sy = ey_of(i);
-                dr += g[i]; jx += sx * g[i]; jy += sy * g[i];
-                sxx += sx * sx * g[i]; sxy += sx * sy * g[i]; syy += sy * sy * g[i];
+            for (int i = 0; i < 9; ++i)
+                for (int j = 0; j < 2; ++j)
+                    if (j < nvalid) f[i * n + k + j] = widen(g[i][j]) + c.shift[i];
+        }
+        if (!o.any()) continue;
+        F2 p[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) p[i] = f2_make(g[i][0], g[i][1]);
+        ExactSum dr(p[0]), jx(p[1]), jy(p[2]);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) dr.plus(p[i]);
+        jx.minus(p[3]); jx.plus(p[5]); jx.minus(p[6]); jx.minus(p[7]); jx.plus(p[8]);
+        jy.minus(p[4]); jy.plus(p[5]); jy.plus(p[6]); jy.minus(p[7]); jy.minus(p[8]);
+        ExactSum sxx(p[1]), sxy(p[5]), syy(p[2]);
+        if (o.second()) {
+            sxx.plus(p[3]); sxx.plus(p[5]); sxx.plus(p[6]); sxx.plus(p[7]); sxx.plus(p[8]);
+            sxy.minus(p[6]); sxy.plus(p[7]); sxy.minus(p[8]);
+            syy.plus(p[4]); syy.plus(p[5]); syy.plus(p[6]); syy.plus(p[7]); syy.plus(p[8]);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            if (j >= nvalid) continue;
+            const float drf = j ? f2_hi(dr.hi) : f2_lo(dr.hi), jxf = j ? f2_hi(jx.hi) : f2_lo(jx.hi);
+            const float jyf = j ? f2_hi(jy.hi) : f2_lo(jy.hi);
+            const float rf = (float)a.rho0 + drf;
+            // the exact sums and the quotients below want ordinary values; the others go the plain way
+            if (!(fabsf(drf) < 1e15f && fabsf(rf) > 1e-15f && fabsf(jxf) < 1e15f && fabsf(jyf) < 1e15f)) {
+                double d[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) d[i] = (double)g[i][j];
+                moments_plain<true>(d, a, o, k + j);
+                continue;
             }
-            // moments of the shift: sum s = rho0, sum xi s = rho0 u_ref,
-            // sum xi_a xi_b s = rho0 (u_ref,a u_ref,b + c_s^2 delta_ab)
-            const double r = a.rho0 + dr;
-            jx += a.rho0 * a.urx;
-            jy += a.rho0 * a.ury;
-            if (rho) rho[k] = r;
-            if (ux) ux[k] = jx / r;
-            if (uy) uy[k] = jy / r;
-            if (pxx) pxx[k] = sxx + a.rho0 * (a.urx * a.urx + 1.0 / 3.0);
-            if (pxy) pxy[k] = sxy + a.rho0 * a.urx * a.ury;
-            if (pyy) pyy[k] = syy + a.rho0 * (a.ury * a.ury + 1.0 / 3.0);
+            const double r = a.rho0 + dr.value(j);
+            if (o.rho) o.rho[k + j] = r;
+            if (o.ux || o.uy) {
+                const double r0 = widen(rcp_approx(rf)), r1 = fma(r0, fma(-r, r0, 1.0), r0);
+                if (o.ux) {
+                    const double q = shifted ? fma(a.rho0, a.urx, jx.value(j)) : jx.value(j), u = q * r1;
+                    o.ux[k + j] = fma(fma(-r, u, q), r1, u);
+                }
+                if (o.uy) {
+                    const double q = shifted ? fma(a.rho0, a.ury, jy.value(j)) : jy.value(j), u = q * r1;
+                    o.uy[k + j] = fma(fma(-r, u, q), r1, u);
+                }
+            }
+            if (o.pxx) o.pxx[k + j] = fma(a.rho0, c.second[0], sxx.value(j));
+            if (o.pxy) o.pxy[k + j] = fma(c.second[1], a.ury, sxy.value(j));
+            if (o.pyy) o.pyy[k + j] = fma(a.rho0, c.second[2], syy.value(j));
         }
     }
 }
@@ -434,7 +585,9 @@ __global__ void halo_kernel(E* buf, FieldArgs a, E* up, E* down, int pack) {
 
 template <typename S>
 cudaError_t init_t(void* buf, const FieldArgs& a, int eq, const double* r, const double* x, const double* y, cudaStream_t s) {
-    init_eq_kernel<S><<<grid_for((long long)a.nx * a.ny), kBlock, 0, s>>>((S*)buf, a, eq, r, x, y);
+    const int grid = grid_for((long long)a.nx * a.ny);
+    if (eq == 4) init_eq_kernel<S><<<grid, kBlock, 0, s>>>((S*)buf, a, equilibrium_consts(a.urx, a.ury), r, x, y);
+    else init_eq_truncated_kernel<S><<<grid, kBlock, 0, s>>>((S*)buf, a, eq, r, x, y);
     return cudaGetLastError();
 }
 template <typename S>
@@ -443,9 +596,17 @@ cudaError_t scatter_t(void* buf, const FieldArgs& a, const double* f, cudaStream
     return cudaGetLastError();
 }
 template <typename S>
-cudaError_t gather_t(const void* buf, const FieldArgs& a, double* f, double* r, double* x, double* y,
-                     double* pxx, double* pxy, double* pyy, cudaStream_t s) {
-    gather_kernel<S><<<grid_for((long long)a.nx * a.ny), kBlock, 0, s>>>((const S*)buf, a, f, r, x, y, pxx, pxy, pyy);
+cudaError_t gather_t(const void* buf, const FieldArgs& a, double* f, const MomentOut& o, cudaStream_t s) {
+    if constexpr (sizeof(S) == 8) {
+        gather_kernel_f64<<<grid_for((long long)a.nx * a.ny), kBlock, 0, s>>>((const double*)buf, a, f, o);
+    } else {
+        GatherConsts c;
+        for (int i = 0; i < 9; ++i) c.shift[i] = shift_of(i, a.rho0, a.urx, a.ury);
+        c.second[0] = std::fma(a.urx, a.urx, 1.0 / 3.0);
+        c.second[1] = a.rho0 * a.urx;
+        c.second[2] = std::fma(a.ury, a.ury, 1.0 / 3.0);
+        gather_kernel<S><<<grid_for((long long)a.ny * ((a.nx + 1) / 2)), kBlock, 0, s>>>((const S*)buf, a, f, o, c);
+    }
     return cudaGetLastError();
 }
 template <typename S>
@@ -508,7 +669,8 @@ cudaError_t launch_scatter(int storage, void* buf, const FieldArgs& a, const dou
 }
 cudaError_t launch_gather(int storage, const void* buf, const FieldArgs& a, double* f, double* rho, double* ux,
                           double* uy, double* pxx, double* pxy, double* pyy, cudaStream_t s) {
-    LBM_DISPATCH(storage, gather_t<S>(buf, a, f, rho, ux, uy, pxx, pxy, pyy, s));
+    const MomentOut o{rho, ux, uy, pxx, pxy, pyy};
+    LBM_DISPATCH(storage, gather_t<S>(buf, a, f, o, s));
 }
 cudaError_t launch_reduce(int storage, const void* buf, const FieldArgs& a, double* partials, unsigned* counter,
                           double* out8, int* status, long long* blowup_step, const CheckArgs& c, cudaStream_t s) {

@@ -14,6 +14,7 @@
 #pragma once
 
 #include "lbm_device.cuh"
+#include "lbm_equilibrium.cuh"
 
 namespace lbm {
 
@@ -23,6 +24,7 @@ struct BatchInstance {   // read-only during a run
     int model;           // lbm::Model
     int pad;
     double ke_ref, ke_factor;   // optional <|u|^2> > ke_factor * ke_ref criterion (ke_ref > 0)
+    EquilibriumConsts eq;       // factors of the shift, for the initial state
 };
 
 struct BatchState {      // updated by the kernel, one per instance

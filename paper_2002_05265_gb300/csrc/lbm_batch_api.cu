@@ -123,20 +123,14 @@ __global__ void batch_init_kernel(S* slab, const BatchInstance* __restrict__ ins
         const long long local = k - node_off[lo];
         const int y = (int)(local / a.nx), x = (int)(local - (long long)y * a.nx);
         S* buf = slab + I.off + (long long)st[lo].cur * 9 * a.plane;
-        const double r = rho[k], vx = ux[k], vy = uy[k], dr = r - a.rho0;
+        S g[9];
+        lbm::equilibrium_node<S>(rho[k], ux[k], uy[k], a.rho0, a.urx, a.ury, I.eq, g);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            const int sx = lbm::ex_of(i), sy = lbm::ey_of(i);
-            // Eq. extendedFeq, product form, minus the shift rho0 phi(u_ref,x) phi(u_ref,y)
-            const double Px = lbm::phi1d(sx, a.urx), Py = lbm::phi1d(sy, a.ury);
-            const double dux = vx - a.urx, sux = vx + a.urx, duy = vy - a.ury, suy = vy + a.ury;
-            const double Dx = sx ? 0.5 * dux * (sux + sx) : -dux * sux;
-            const double Dy = sy ? 0.5 * duy * (suy + sy) : -duy * suy;
-            const double g = Px * Py * dr + r * (Px * Dy + Dx * (Py + Dy));
-            int xs = x - sx, ys = y - sy;
+            int xs = x - lbm::ex_of(i), ys = y - lbm::ey_of(i);
             xs = xs < 0 ? xs + a.nx : (xs >= a.nx ? xs - a.nx : xs);
             ys = ys < 0 ? ys + a.ny : (ys >= a.ny ? ys - a.ny : ys);
-            buf[(long long)i * a.plane + (long long)ys * a.pitch + xs] = lbm::Conv<S>::from_double(g);
+            buf[(long long)i * a.plane + (long long)ys * a.pitch + xs] = g[i];
         }
     }
 }
@@ -256,6 +250,7 @@ int lbm_batch_create(lbm_batch** out, int n, const lbm_instance_desc* desc, int 
         I.pad = 0;
         I.ke_ref = d.ke_ref;
         I.ke_factor = d.ke_factor;
+        I.eq = lbm::equilibrium_consts(d.ux_ref, d.uy_ref);
         off = (off + 127) / 128 * 128;   // 256-byte aligned or better for every storage type
         I.off = off;
         off += 2 * 9 * I.a.plane;
