@@ -390,7 +390,8 @@ int lbm_batch_run(lbm_batch* b, long long target_steps, int check_every, double 
 int lbm_batch_status(lbm_batch* b, int* status, long long* blowup_step, long long* steps, double* diag4);
 /* Canonical pre-collision populations of one instance as FP64 [9][ny][nx]. */
 int lbm_batch_get_populations(lbm_batch* b, int index, double* f);
-/* Kernel shape: `vec` x-nodes per thread and `block` threads per CTA.  autotune times every
+/* Kernel shape: `vec` x-nodes per thread (of the steps that check, and of FP64) and `block` threads
+ * per CTA (one CTA advances an instance; by default 512, FP64 256).  autotune times every
  * instantiated shape for `trial_steps` steps from the current state (restoring the state
  * after each trial), keeps the fastest and reports it. */
 int lbm_batch_set_shape(lbm_batch* b, int vec, int block);

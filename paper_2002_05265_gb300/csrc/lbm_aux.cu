@@ -171,6 +171,7 @@ __device__ __forceinline__ void moments_plain(const double (&g)[9], const FieldA
 
 // FP64 storage: one node per thread.
 __global__ void gather_kernel_f64(const double* buf, FieldArgs a, double* f, MomentOut o) {
+    if (a.which && *a.which) buf += a.other;
     const long long n = (long long)a.nx * a.ny;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const int y = (int)(k / a.nx), x = (int)(k - (long long)y * a.nx);
@@ -198,6 +199,7 @@ struct GatherConsts {
 };
 template <typename S>
 __global__ void __launch_bounds__(kBlock) gather_kernel(const S* buf, FieldArgs a, double* f, MomentOut o, GatherConsts c) {
+    if (a.which && *a.which) buf += a.other;
     const long long n = (long long)a.nx * a.ny;
     const int lane = threadIdx.x & 31, nseg = (a.nx + 1) / 2;
     const bool shifted = a.urx != 0.0 || a.ury != 0.0;

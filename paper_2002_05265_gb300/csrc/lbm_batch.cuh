@@ -2,10 +2,14 @@
 // with its own collision model, relaxation rates and blow-up state, advanced by ONE
 // persistent launch (the numerical-stability study of Sec. 5b run as a batch).
 //
+// Stepping: FP32 and 16-bit instances take the time-fused marches of lbm_march.cuh between checks
+// (four steps per read and write of the instance, the collision in two-wide FP32 instructions);
+// the step that checks, and FP64, sweep the instance's vector segments once per step.
+//
 // Scheduling: the grid holds as many CTAs as the GPU keeps resident.  Each CTA repeatedly
 // claims the next instance from a global counter (instances ordered largest first), and
-// advances that instance alone from its current step to the target step: every time step is
-// one sweep of the CTA over the instance's vector segments followed by __syncthreads(), which
+// advances that instance alone from its current step to the target step: every step or block of
+// fused steps is one sweep of the CTA over the instance followed by __syncthreads(), which
 // is the per-instance barrier (an instance never spans CTAs, so no inter-CTA waits exist and
 // nothing can deadlock).  Every `check_every` steps the sweep also accumulates the blow-up
 // diagnostics of the pre-collision state in FP64 (perturbation energy, kinetic energy,
@@ -15,6 +19,7 @@
 
 #include "lbm_device.cuh"
 #include "lbm_equilibrium.cuh"
+#include "lbm_march.cuh"
 
 namespace lbm {
 
@@ -38,8 +43,49 @@ struct BatchState {      // updated by the kernel, one per instance
 
 constexpr double kPertFloor = 1e-20;   // <|u - u_ref|^2> below this counts as "no perturbation"
 
+// Time steps `t` .. `t + n` of one instance without a check, fused as in lbm_march.cuh: the CTA's
+// warps share its strips and bands of rows, and a block of up to four steps ends at a barrier.
+// Measured on 1024 instances of 32..256 squared for 1000 steps (FP32): 245 -> 147 ms (87 -> 147
+// GLUPS) with 16 warps a CTA, 162 ms with 8 (200 instances: 58 and 105 ms, hence the default); the
+// unrolled form, whose code outgrows the instruction cache here, 225 ms.  What bounds it: 84 % of the
+// columns and 84 % of the rows that are marched are kept, the rest of the time is the FP32 pipe's.
+template <int MODEL, typename S, int BLOCK, bool PAIRS>
+__device__ __forceinline__ int batch_march(S* buf0, S* buf1, int cur, int n, const StepArgs& a, const Consts<F2>& c) {
+    constexpr int WARPS = BLOCK / 32, TMAX = MarchForm<S>::TMAX;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    extern __shared__ __align__(16) unsigned char march_smem[];
+    auto* own = reinterpret_cast<typename MarchPair<S>::type*>(march_smem) + warp * march_warp_rows<TMAX, true> * 32 + lane;
+    const int blocks = (n + TMAX - 1) / TMAX;
+    // bands: rounds of the warps times rows of a march, its t - 1 redundant rows included
+    const int strips = (a.nx + march_width(TMAX) - 1) / march_width(TMAX);
+    int bands = 1, least = 1 << 30;
+    for (int b = 1; b <= 2 * WARPS; ++b) {
+        const int cost = (strips * b + WARPS - 1) / WARPS * ((a.ny + b - 1) / b + TMAX - 1);
+        if (cost < least) {
+            least = cost;
+            bands = b;
+        }
+    }
+#pragma unroll 1
+    for (int k = 0; k < blocks; ++k) {
+        const int t = n / blocks + (k < n % blocks ? 1 : 0);
+        const int tasks = (a.nx + march_width(t) - 1) / march_width(t) * bands;
+#pragma unroll 1
+        for (int task = warp; task < tasks; task += WARPS) {
+            const int strip = task / bands, band = task - strip * bands;
+            const int y0 = (int)((long long)band * a.ny / bands), y1 = (int)((long long)(band + 1) * a.ny / bands);
+            if (y0 == y1) continue;
+            march<MODEL, S, true, TMAX, PAIRS, true>(cur ? buf1 : buf0, cur ? buf0 : buf1, a.nx, a.ny, a.pitch, a.plane, c,
+                                                     t, strip * march_width(t), y0, y1, lane, own);
+        }
+        cur ^= 1;
+        __syncthreads();   // the block's stores are visible to the CTA before the next block reads
+    }
+    return cur;
+}
+
 template <int MODEL, typename S, int VEC, int BLOCK>
-__device__ __forceinline__ void batch_instance_loop(S* __restrict__ buf0, S* __restrict__ buf1, const StepArgs& a,
+__device__ __forceinline__ void batch_instance_loop(S* buf0, S* buf1, const StepArgs& a,
                                                     const BatchInstance& I, BatchState& st, long long target,
                                                     int check_every, double growth, double (*s_red)[4],
                                                     int* s_stop) {
@@ -47,6 +93,7 @@ __device__ __forceinline__ void batch_instance_loop(S* __restrict__ buf0, S* __r
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned total = (unsigned)a.ny * (unsigned)a.nseg;
     const Consts<T> c = make_consts<T>(a);
+    const Consts<F2> cp = make_consts_f2(a.cf);
     long long t = st.steps;
     int cur = st.cur;
     const double nodes = (double)a.nx * (double)a.ny;
@@ -89,9 +136,17 @@ __device__ __forceinline__ void batch_instance_loop(S* __restrict__ buf0, S* __r
                 }
                 *s_stop = blown ? 1 : 0;
             }
-        } else {
+        } else if constexpr (sizeof(S) == 8) {
             for (unsigned base = threadIdx.x & ~31u; base < total; base += BLOCK)
                 step_segment<MODEL, 4, S, VEC, false, true>(src, dst, a, c, base + lane, total, lane, dg);
+        } else {
+            // up to the next check
+            const long long next = check_every > 0 ? (t / check_every + 1) * (long long)check_every : target;
+            const int n = (int)min(min(next, target) - t, (long long)(1 << 20));
+            if (a.nx % 2 == 0) cur = batch_march<MODEL, S, BLOCK, true>(buf0, buf1, cur, n, a, cp);
+            else cur = batch_march<MODEL, S, BLOCK, false>(buf0, buf1, cur, n, a, cp);
+            t += n;
+            continue;
         }
         __syncthreads();   // step t complete (stores visible to the CTA) before step t + 1 reads
         cur ^= 1;
@@ -105,7 +160,7 @@ __device__ __forceinline__ void batch_instance_loop(S* __restrict__ buf0, S* __r
 }
 
 template <typename S, int VEC, int BLOCK>
-__global__ void __launch_bounds__(BLOCK) batch_kernel(S* slab, const BatchInstance* __restrict__ inst,
+__global__ void __launch_bounds__(BLOCK, sizeof(S) == 8 ? 1 : 512 / BLOCK) batch_kernel(S* slab, const BatchInstance* __restrict__ inst,
                                                       BatchState* state, const int* __restrict__ order, int n,
                                                       int* queue, long long target, int check_every, double growth) {
     __shared__ int s_id;

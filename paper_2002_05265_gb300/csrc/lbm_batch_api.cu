@@ -75,9 +75,15 @@ const void* pick_batch_kernel(int storage, int vec, int block) {
     }
 }
 
+// dynamic shared memory of a batch kernel: the fused marches' of its warps (none for FP64)
+int batch_smem(int storage, int block) {
+    if (storage == LBM_F64) return 0;
+    return block / 32 * (storage == LBM_F32 ? lbm::march_smem_bytes<float, true> : lbm::march_smem_bytes<__half, true>);
+}
+
 void default_shape(int storage, int* vec, int* block) {
     *vec = 16 / lbm::storage_bytes(storage);
-    *block = 256;
+    *block = storage == LBM_F64 ? 256 : 512;
 }
 
 bool is_device_ptr(const void* p) {
@@ -95,7 +101,9 @@ int set_shape(lbm_batch* b, int vec, int block) {
     int dev = 0, sms = 0, per_sm = 0;
     LBM_BCK(b, cudaGetDevice(&dev));
     LBM_BCK(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    LBM_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, 0));
+    const int smem = batch_smem(b->storage, block);
+    LBM_BCK(b, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    LBM_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     if (per_sm < 1) return berr(b, LBM_ERR_UNSUPPORTED, "batch kernel cannot be resident");
     b->kernel = k;
     b->vec = vec;
@@ -184,7 +192,7 @@ int record_run(lbm_batch* b, long long target, int check_every, double growth) {
         int ce = check_every;
         double gr = growth;
         void* args[] = {&slab, &di, &ds, &dord, &n, &dq, &tg, &ce, &gr};
-        cudaLaunchKernel(b->kernel, dim3(b->grid), dim3(b->block), args, 0, cap);
+        cudaLaunchKernel(b->kernel, dim3(b->grid), dim3(b->block), args, batch_smem(b->storage, b->block), cap);
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(cap, &graph);
         if (e == cudaSuccess) {
@@ -381,15 +389,14 @@ int lbm_batch_status(lbm_batch* b, int* status, long long* blowup_step, long lon
 int lbm_batch_get_populations(lbm_batch* b, int index, double* f) {
     if (!b || !f || index < 0 || index >= b->n)
         return b ? berr(b, LBM_ERR_INVALID_ARG, "bad instance index or null output") : LBM_ERR_INVALID_ARG;
-    BatchState s;
-    LBM_BCK(b, cudaMemcpyAsync(&s, b->d_state + index, sizeof(s), cudaMemcpyDeviceToHost, b->stream));
-    LBM_BCK(b, cudaStreamSynchronize(b->stream));
     const BatchInstance& I = b->inst[index];
     lbm::FieldArgs a;
     a.nx = I.a.nx; a.ny = I.a.ny; a.pitch = I.a.pitch; a.plane = I.a.plane; a.rho0 = I.a.rho0;
     a.urx = I.a.urx; a.ury = I.a.ury;
-    const char* base = static_cast<const char*>(b->slab) +
-                       (size_t)(I.off + (long long)s.cur * 9 * I.a.plane) * lbm::storage_bytes(b->storage);
+    // the kernel reads which of the two buffers is current: no round trip to the host before it
+    a.which = &b->d_state[index].cur;
+    a.other = 9 * I.a.plane;
+    const char* base = static_cast<const char*>(b->slab) + (size_t)I.off * lbm::storage_bytes(b->storage);
     const size_t n = (size_t)I.a.nx * I.a.ny;
     double* dst = f;
     double* tmp = nullptr;
@@ -421,7 +428,7 @@ int lbm_batch_get_shape(const lbm_batch* b, int* vec, int* block, int* grid) {
 
 int lbm_batch_autotune(lbm_batch* b, long long trial_steps, int check_every, int* vec, int* block, double* best_ms) {
     if (!b || trial_steps < 1 || check_every < 0) return b ? berr(b, LBM_ERR_INVALID_ARG, "bad trial") : LBM_ERR_INVALID_ARG;
-    static const int cand[][2] = {{2, 128}, {2, 256}, {2, 512}, {4, 128}, {4, 256}, {4, 512}, {8, 128}, {8, 256}};
+    static const int cand[][2] = {{2, 128}, {2, 256}, {2, 512}, {4, 128}, {4, 256}, {4, 512}, {8, 128}, {8, 256}, {8, 512}};
     // save the state, time each shape from it, restore it after every trial
     std::vector<BatchState> s0(b->n);
     LBM_BCK(b, cudaMemcpyAsync(s0.data(), b->d_state, sizeof(BatchState) * b->n, cudaMemcpyDeviceToHost, b->stream));

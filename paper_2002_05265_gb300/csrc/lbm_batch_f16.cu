@@ -5,6 +5,7 @@
 
 namespace lbm {
 const void* batch_kernel_f16(int vec, int block) {
+    if (vec == 8 && block == 512) return (const void*)batch_kernel<__half, 8, 512>;
     if (vec == 8 && block == 256) return (const void*)batch_kernel<__half, 8, 256>;
     if (vec == 8 && block == 128) return (const void*)batch_kernel<__half, 8, 128>;
     if (vec == 4 && block == 256) return (const void*)batch_kernel<__half, 4, 256>;

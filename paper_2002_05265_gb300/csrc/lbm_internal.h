@@ -57,6 +57,8 @@ struct FieldArgs {
     long long plane;
     double rho0;         // shift s_i = rho0 phi(u_ref,x) phi(u_ref,y)
     double urx, ury;
+    const int* which = nullptr;   // launch_gather: reads the buffer + other elements where *which != 0
+    long long other = 0;
 };
 // f(x) = f^eq(rho(x), u(x)) (eq_order 2 or 4), scattered so the next pull gathers it.
 cudaError_t launch_init_eq(int storage, void* buf, const FieldArgs& a, int eq_order,

@@ -141,7 +141,10 @@ struct MarchArgs {
 };
 
 __device__ __forceinline__ F2 f2_of(float2 v) { return f2_make(v.x, v.y); }
-__device__ __forceinline__ Consts<F2> make_consts_f2(const float2* t) {
+__device__ __forceinline__ F2 f2_of(float v) { return f2_make(v, v); }
+// from a constant table, or one with every entry twice
+template <typename E>
+__device__ __forceinline__ Consts<F2> make_consts_f2(const E* t) {
     Consts<F2> c;
     c.w = f2_of(t[0]); c.w3 = f2_of(t[1]); c.w4 = f2_of(t[2]); c.rho0 = f2_of(t[3]);
     c.urx = f2_of(t[4]); c.ury = f2_of(t[5]);

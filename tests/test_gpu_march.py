@@ -85,3 +85,32 @@ def test_fused_group_of_unequal_lattices(L, models, storage):
     L.lbm_group_destroy(g)
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("check", [0, 7, 50])
+def test_fused_batch_equals_lattices(L, storage, check):
+    """Instances of a sweep, fused between checks, against lattices of the register-staged kernels
+    stored around the same mean flow: narrow, odd, wide and flat ones, every model, bit for bit."""
+    shapes = [(32, 33), (57, 3), (61, 140), (64, 64), (113, 200), (256, 17), (3, 256), (200, 35)]
+    u = [(0.05 + 0.01 * k, 0.02 - 0.01 * k) for k in range(len(shapes))]
+    descs = [dict(nx=nx, ny=ny, model=m, rates=(1.9, 1.3, 0.9), ux_ref=a, uy_ref=b)
+             for (nx, ny), m, (a, b) in zip(shapes, MODELS, u)]
+    fields = [_fields(nx, ny, nx + ny) for nx, ny in shapes]
+    b = L.lbm_batch_create(descs, storage=L.STORAGES[storage])
+    L.lbm_batch_init_equilibrium(b, *[torch.cat([f[i].flatten() for f in fields]) for i in range(3)])
+    for target in (41, 42, 103):
+        L.lbm_batch_run(b, target, check_every=check, growth=1e12)
+    status, _, steps, _ = L.lbm_batch_status(b, len(descs))
+    assert list(status) == [0] * len(descs) and list(steps) == [103] * len(descs)
+    for k, ((nx, ny), m) in enumerate(zip(shapes, MODELS)):
+        lat = L.Lattice(nx, ny, m, (1.9, 1.3, 0.9), storage=L.STORAGES[storage])
+        lat.set_shift_velocity(*u[k])
+        lat.set_kernel_path(L.LBM_PATH_VECTOR)
+        lat.init_equilibrium(*fields[k])
+        lat.step(103)
+        got = torch.empty((9, ny, nx), dtype=torch.float64, device="cuda")
+        L.lbm_batch_get_populations(b, k, got)
+        assert torch.equal(got, _state(lat)), (m, nx, ny)
+        lat.close()
+    L.lbm_batch_destroy(b)
