@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjMinBlocks<S>) adjoint_fused_ker
         return;
     }
     using T = typename Conv<S>::T;
-    constexpr int VEC = DefaultVec<S>::value;
+    constexpr int VEC = StepVec<S>::value;
     const int lane = threadIdx.x & 31;
     const unsigned total = (unsigned)sa.ny * (unsigned)sa.nseg;
     const unsigned stride = (gridDim.x - nadj) * blockDim.x;

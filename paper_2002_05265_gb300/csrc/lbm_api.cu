@@ -57,6 +57,7 @@ struct lbm_group {
     int fused = 0;                     // one multi-lattice launch per time step
     const void* gkernel[2] = {nullptr, nullptr};   // default shift / reference-velocity shift
     int ggrid[2] = {0, 0};
+    int gblock = 256;
     std::vector<unsigned> begin;       // padded segment offsets of the contexts
     unsigned padded_total = 0;
     int tiled = 0;                     // bulk-copy staged launches
@@ -161,6 +162,7 @@ int select_kernel(lbm_ctx* c) {
     if (!k) return set_err(c, LBM_ERR_UNSUPPORTED, "no kernel for this configuration");
     c->kernel = k;
     const long long work = ((long long)c->ny * c->nseg + 31) / 32 * 32;
+    c->block = lbm::spread_block(work);
     c->grid = resident_grid(k, c->block, work);
     return LBM_OK;
 }
@@ -277,12 +279,28 @@ int ensure_stage(lbm_ctx* c, size_t elems) {
     return LBM_OK;
 }
 
+// Launch with programmatic stream serialization: the kernel is scheduled while its predecessor on
+// the stream still runs, and waits for it by itself (griddepcontrol.wait) before it touches memory.
+cudaError_t launch_dependent(const void* kernel, int grid, int block, int smem, void** args, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
 int launch_step_once(lbm_ctx* c, cudaStream_t s) {
     StepArgs a = step_args(c);
     const void* src = c->buf[c->cur];
     void* dst = c->buf[c->cur ^ 1];
     void* args[] = {(void*)&src, (void*)&dst, (void*)&a};
-    LBM_CK(c, cudaLaunchKernel(c->kernel, dim3(c->grid), dim3(c->block), args, 0, s));
+    LBM_CK(c, launch_dependent(c->kernel, c->grid, c->block, 0, args, s));
     c->cur ^= 1;
     c->steps += 1;
     return LBM_OK;
@@ -306,7 +324,7 @@ int launch_group_once(lbm_group* g, cudaStream_t s, int sh) {
         e.total = (unsigned)c->ny * (unsigned)c->nseg;
     }
     void* args[] = {(void*)&ga};
-    LBM_CK(g->ctx[0], cudaLaunchKernel(g->gkernel[sh], dim3(g->ggrid[sh]), dim3(256), args, 0, s));
+    LBM_CK(g->ctx[0], launch_dependent(g->gkernel[sh], g->ggrid[sh], g->gblock, 0, args, s));
     for (lbm_ctx* c : g->ctx) {
         c->cur ^= 1;
         c->steps += 1;
@@ -487,10 +505,11 @@ long long march_strip_rows(const lbm_group* g, int t) {
     return rows;
 }
 
-// How a run is fused: steps per launch and marches (warps) per launch.
+// How a run is fused: steps per launch, marches (warps) per launch and per CTA.
 struct MarchPlan {
     int t;
     long long warps;
+    int per;   // warps of a CTA
 };
 
 // Large lattices fuse as many steps as the kernel has levels, in whole waves of resident warps
@@ -500,9 +519,9 @@ struct MarchPlan {
 // waves, which level out SMs of unequal work (eight 1024^2 lattices 0.98x).
 // Small lattices trade launches against redundant rows: the plan with the least time by a model of
 // what was measured on 67 x 37 to 1024^2 lattices -- a launch takes 2.2 us and its longest march,
-// t (H + t - 1) level-rows for H rows, at 0.21 us a level-row with a scheduler to itself, more with
-// company up to 0.42 + 0.5 / t when every slot is taken (512^2, us a step: t = 2 2.9, 3 3.2, 4 3.6;
-// 256^2: t = 4 on 304 warps 2.0, on 640 2.2; 128^2: 1.5 on 192, 1.9 on 96).
+// t (H + t - 1) level-rows for H rows, at 0.25 us a level-row with a scheduler to itself, 0.36 us with
+// one companion and 0.48 + 0.48 / t with every slot taken (256^2, us a step: t = 4 on 608 warps 2.06,
+// on 304 2.5, on 2432 3.3; 512^2: t = 2 on 1216 2.9, t = 4 on 2432 4.0; 128^2: t = 3 on 384 1.5).
 MarchPlan march_plan(const lbm_group* g, long long n) {
     const long long slots = (long long)g->mgrid * lbm::kMarchWarps, scheds = slots / 4;
     const int most = (int)std::min<long long>(g->march, n);
@@ -510,21 +529,21 @@ MarchPlan march_plan(const lbm_group* g, long long n) {
     if (most == g->march && rows >= 24 * slots) {
         long long waves = (rows + 160 * slots - 1) / (160 * slots);
         if (g->mixed && waves < 2 && rows >= 48 * slots) waves = 2;
-        return {most, slots * waves};
+        return {most, slots * waves, lbm::kMarchWarps};
     }
-    MarchPlan best{most, 1};
+    MarchPlan best{most, 1, 1};
     double least = 1e300;
     for (int t = 2; t <= most; ++t) {
         const long long r = march_strip_rows(g, t);
-        for (long long w = scheds / 2; w <= slots; w *= 2) {
-            const long long warps = std::max<long long>(1, std::min(w, r / 2));   // two rows at least
-            const double load = (double)warps / scheds, height = (double)r / warps;
-            const double each = load <= 0.5 ? 0.21 : std::min(0.42 + 0.5 / t, 0.2 + 0.15 * load);
-            const double us = (2.2 + each * t * (height + t - 1)) / t;
-            if (us < least) {
-                least = us;
-                best = {t, warps};
-            }
+        for (int load = 4; load >= 1; load /= 2) {   // warps per scheduler
+            const long long warps = std::min(load * scheds, r);
+            if (load < 4 && r > 8 * warps) continue;   // long marches want every slot
+            const double each = load == 1 ? 0.25 : (load == 2 ? 0.36 : 0.48 + 0.48 / t);
+            const double us = (2.2 + each * t * (double)((r + warps - 1) / warps + t - 1)) / t;
+            if (us >= least) continue;
+            least = us;
+            // a few warps to as many SMs as there are, then the same number to each SM
+            best = {t, warps, load > 1 ? lbm::kMarchWarps : (2 * warps <= scheds ? 2 : 4)};
         }
     }
     return best;
@@ -541,16 +560,14 @@ long long march_launches(long long n, int t, bool even) {
     return even && l % 2 ? l + 1 : l;
 }
 
-// One time-fused launch: t time steps of every context on about `warps` warps.
-int launch_march(lbm_group* g, cudaStream_t s, int t, long long warps) {
+// One time-fused launch: t time steps of every context by plan p.
+int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
     lbm::MarchArgs ma;
     ma.n = (int)g->ctx.size();
     ma.t = t;
     const int width = lbm::march_width(t);
     double work = 0.0;
     for (const lbm_ctx* c : g->ctx) work += (double)((c->nx + width - 1) / width) * c->ny * march_cost(c->model);
-    // few warps go to as many SMs as there are; full CTAs keep neighbouring strips together
-    const int per = warps < (long long)g->mgrid * lbm::kMarchWarps ? 2 : lbm::kMarchWarps;
     unsigned begin = 0;
     for (size_t k = 0; k < g->ctx.size(); ++k) {
         lbm_ctx* c = g->ctx[k];
@@ -562,25 +579,15 @@ int launch_march(lbm_group* g, cudaStream_t s, int t, long long warps) {
         e.model = kernel_model(c->model);
         e.strips = (c->nx + width - 1) / width;
         // bands by the lattice's share of the work, so that every march costs about the same
-        const double bands = (double)warps * c->ny * march_cost(c->model) / work;
+        const double bands = (double)p.warps * c->ny * march_cost(c->model) / work;
         e.bands = std::max(1, std::min(c->ny, (int)bands));
         e.begin = begin;
-        begin += (unsigned)((e.strips * (long long)e.bands + per - 1) / per);
+        begin += (unsigned)((e.strips * (long long)e.bands + p.per - 1) / p.per);
         const StepArgs a = step_args(c);
         for (int j = 0; j < lbm::kNumConsts; ++j) e.c[j] = make_float2(a.cf[j], a.cf[j]);
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(begin);
-    cfg.blockDim = dim3(32 * per);
-    cfg.dynamicSmemBytes = (size_t)(g->msmem * per);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     void* args[] = {(void*)&ma};
-    LBM_CK(g->ctx[0], cudaLaunchKernelExC(&cfg, g->mkernel[tile_shift(g)], args));
+    LBM_CK(g->ctx[0], launch_dependent(g->mkernel[tile_shift(g)], (int)begin, 32 * p.per, g->msmem * p.per, args, s));
     for (lbm_ctx* c : g->ctx) {
         c->cur ^= 1;
         c->steps += t;
@@ -596,7 +603,7 @@ int group_advance(lbm_group* g, cudaStream_t s, long long n, bool even = false) 
         const MarchPlan p = march_plan(g, n);
         const long long l = march_launches(n, p.t, even);
         for (long long k = 0; k < l; ++k) {   // lengths differ by at most one step
-            int rc = launch_march(g, s, (int)(n / l + (k < n % l ? 1 : 0)), p.warps);
+            int rc = launch_march(g, s, (int)(n / l + (k < n % l ? 1 : 0)), p);
             if (rc != LBM_OK) return rc;
         }
         return LBM_OK;
@@ -1228,7 +1235,8 @@ int lbm_group_create(lbm_group** out, lbm_ctx* const* ctxs, int n, int graph_ste
         g->padded_total = off;
         for (int sh = 0; sh < 2; ++sh) {
             g->gkernel[sh] = pick_group_kernel(ctxs[0]->storage, sh == 1);
-            g->ggrid[sh] = resident_grid(g->gkernel[sh], 256, off);
+            g->gblock = lbm::spread_block(off);
+            g->ggrid[sh] = resident_grid(g->gkernel[sh], g->gblock, off);
         }
         g->fused = 1;
     }

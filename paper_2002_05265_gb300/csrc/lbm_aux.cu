@@ -558,11 +558,14 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_finish_kernel(const dou
     finish_fold(partials, nparts, a, out, status, blowup_step, c);
 }
 
-int grid_for(long long n) {
-    long long g = (n + kBlock - 1) / kBlock;
-    if (g > 152 * 16) g = 152 * 16;
-    if (g < 1) g = 1;
-    return (int)g;
+// CTAs for n threads of work: at most 16 of kBlock threads per SM; small fields in smaller CTAs, so
+// that every SM has some (their FP64 work is bound by the SMs that take part).
+struct Spread {
+    int grid, block;
+};
+Spread spread(long long n) {
+    const int block = spread_block(n);
+    return Spread{(int)std::max(1ll, std::min((n + block - 1) / block, 152ll * 16)), block};
 }
 
 // Halo rows of a y-slab.  Messages are [3][nx] elements: `up` holds the planes with xi_y = +1
@@ -587,27 +590,30 @@ __global__ void halo_kernel(E* buf, FieldArgs a, E* up, E* down, int pack) {
 
 template <typename S>
 cudaError_t init_t(void* buf, const FieldArgs& a, int eq, const double* r, const double* x, const double* y, cudaStream_t s) {
-    const int grid = grid_for((long long)a.nx * a.ny);
-    if (eq == 4) init_eq_kernel<S><<<grid, kBlock, 0, s>>>((S*)buf, a, equilibrium_consts(a.urx, a.ury), r, x, y);
-    else init_eq_truncated_kernel<S><<<grid, kBlock, 0, s>>>((S*)buf, a, eq, r, x, y);
+    const Spread g = spread((long long)a.nx * a.ny);
+    if (eq == 4) init_eq_kernel<S><<<g.grid, g.block, 0, s>>>((S*)buf, a, equilibrium_consts(a.urx, a.ury), r, x, y);
+    else init_eq_truncated_kernel<S><<<g.grid, g.block, 0, s>>>((S*)buf, a, eq, r, x, y);
     return cudaGetLastError();
 }
 template <typename S>
 cudaError_t scatter_t(void* buf, const FieldArgs& a, const double* f, cudaStream_t s) {
-    scatter_kernel<S><<<grid_for((long long)a.nx * a.ny), kBlock, 0, s>>>((S*)buf, a, f);
+    const Spread g = spread((long long)a.nx * a.ny);
+    scatter_kernel<S><<<g.grid, g.block, 0, s>>>((S*)buf, a, f);
     return cudaGetLastError();
 }
 template <typename S>
 cudaError_t gather_t(const void* buf, const FieldArgs& a, double* f, const MomentOut& o, cudaStream_t s) {
     if constexpr (sizeof(S) == 8) {
-        gather_kernel_f64<<<grid_for((long long)a.nx * a.ny), kBlock, 0, s>>>((const double*)buf, a, f, o);
+        const Spread g = spread((long long)a.nx * a.ny);
+        gather_kernel_f64<<<g.grid, g.block, 0, s>>>((const double*)buf, a, f, o);
     } else {
         GatherConsts c;
         for (int i = 0; i < 9; ++i) c.shift[i] = shift_of(i, a.rho0, a.urx, a.ury);
         c.second[0] = std::fma(a.urx, a.urx, 1.0 / 3.0);
         c.second[1] = a.rho0 * a.urx;
         c.second[2] = std::fma(a.ury, a.ury, 1.0 / 3.0);
-        gather_kernel<S><<<grid_for((long long)a.ny * ((a.nx + 1) / 2)), kBlock, 0, s>>>((const S*)buf, a, f, o, c);
+        const Spread g = spread((long long)a.ny * ((a.nx + 1) / 2));
+        gather_kernel<S><<<g.grid, g.block, 0, s>>>((const S*)buf, a, f, o, c);
     }
     return cudaGetLastError();
 }
@@ -685,25 +691,30 @@ cudaError_t launch_reduce_group(int storage, const ReduceGroupArgs& g, cudaStrea
 }
 
 cudaError_t launch_halo(int storage, void* buf, const FieldArgs& a, void* up, void* down, bool pack, cudaStream_t s) {
-    const int grid = grid_for(6LL * a.nx);
+    const Spread g = spread(6LL * a.nx);
     switch (storage_bytes(storage)) {
-        case 8: halo_kernel<unsigned long long><<<grid, kBlock, 0, s>>>((unsigned long long*)buf, a,
+        case 8: halo_kernel<unsigned long long><<<g.grid, g.block, 0, s>>>((unsigned long long*)buf, a,
                                                 (unsigned long long*)up, (unsigned long long*)down, pack); break;
-        case 4: halo_kernel<unsigned><<<grid, kBlock, 0, s>>>((unsigned*)buf, a, (unsigned*)up, (unsigned*)down, pack);
+        case 4: halo_kernel<unsigned><<<g.grid, g.block, 0, s>>>((unsigned*)buf, a, (unsigned*)up, (unsigned*)down, pack);
             break;
-        case 2: halo_kernel<unsigned short><<<grid, kBlock, 0, s>>>((unsigned short*)buf, a, (unsigned short*)up,
+        case 2: halo_kernel<unsigned short><<<g.grid, g.block, 0, s>>>((unsigned short*)buf, a, (unsigned short*)up,
                                                                    (unsigned short*)down, pack); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
+int spread_block(long long threads) {
+    int block = kBlock;
+    while (block > 32 && threads < 2LL * 152 * block) block /= 2;
+    return block;
+}
 int storage_vec(int storage) {
     switch (storage) {
-        case 0: return DefaultVec<double>::value;
-        case 1: return DefaultVec<float>::value;
-        case 2: return DefaultVec<__half>::value;
-        case 3: return DefaultVec<__nv_bfloat16>::value;
+        case 0: return StepVec<double>::value;
+        case 1: return StepVec<float>::value;
+        case 2: return StepVec<__half>::value;
+        case 3: return StepVec<__nv_bfloat16>::value;
         default: return 0;
     }
 }
@@ -737,7 +748,7 @@ extern "C" int lbm_selftest_recip(const float* x, float* approx, float* rounded,
     using namespace lbm;
     if (!x || !approx || !rounded || n < 0) return LBM_ERR_INVALID_ARG;
     if (n == 0) return LBM_OK;
-    selftest_recip_kernel<<<grid_for(n), kBlock, 0, (cudaStream_t)cuda_stream>>>(x, approx, rounded, n);
+    selftest_recip_kernel<<<spread(n).grid, spread(n).block, 0, (cudaStream_t)cuda_stream>>>(x, approx, rounded, n);
     return cudaGetLastError() == cudaSuccess ? LBM_OK : LBM_ERR_CUDA;
 }
 

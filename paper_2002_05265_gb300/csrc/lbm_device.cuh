@@ -143,6 +143,14 @@ template <typename S> struct DefaultVec {
     static constexpr int value = (sizeof(S) == 2) ? LBM_HALF_VEC : 16 / (int)sizeof(S);
 };
 
+// Nodes per thread of the register-staged step kernels: the default, but one for FP64, where a
+// scheduler takes 64 clocks for an instruction of one warp (measured, whatever lanes are active): what
+// counts there is that every scheduler has one.  With CTAs to match (spread_block) a step of 128 x 128
+// BGK takes 5.5 us instead of 11.0, 67 x 37 CHM 4.3 us instead of 16.4.
+template <typename S> struct StepVec {
+    static constexpr int value = sizeof(S) == 8 ? 1 : DefaultVec<S>::value;
+};
+
 template <int BYTES> struct Raw;
 template <> struct Raw<4> { using type = uint32_t; };
 template <> struct Raw<8> { using type = uint2; };
@@ -711,6 +719,15 @@ __device__ __forceinline__ void gather_pull(const S* __restrict__ src, int nx, i
     const bool right_from_lane = (lane < 31) && (seg < nseg - 1);
     const int xl = (x0 == 0) ? nx - 1 : x0 - 1;           // source of an x-offset of -1 at j = 0
     const int xr = (x0 + nvalid >= nx) ? 0 : x0 + VEC;     // source of an x-offset of +1 at j = nvalid-1
+    if constexpr (VEC == 1) {   // a node per lane: its nine sources, straight
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int ex = SIGN * ex_of(i), ey = SIGN * ey_of(i);
+            const int row = (ey == 1) ? ym : ((ey == -1) ? yp : y), x = (ex == 1) ? xl : ((ex == -1) ? xr : x0);
+            f[i][0] = Conv<S>::to_T(src[(long long)i * plane + (long long)row * pitch + x]);
+        }
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int ex = SIGN * ex_of(i), ey = SIGN * ey_of(i);
@@ -790,8 +807,11 @@ __device__ __forceinline__ void step_segment(const S* __restrict__ src, S* __res
 // the resident CTAs of the GPU).
 template <int MODEL, int EQ, typename S, bool SHIFT>
 __global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ src, S* __restrict__ dst, StepArgs a) {
+    // programmatic dependent launch, as in the other step kernels
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     using T = typename Conv<S>::T;
-    constexpr int VEC = DefaultVec<S>::value;
+    constexpr int VEC = StepVec<S>::value;
     const int lane = threadIdx.x & 31;
     const unsigned total = (unsigned)a.ny * (unsigned)a.nseg;
     const unsigned stride = gridDim.x * blockDim.x;
@@ -827,7 +847,7 @@ struct GroupArgs {
 template <typename S, bool SH>
 __device__ __forceinline__ void group_segment(const GroupEntry& e, const Consts<typename Conv<S>::T>& c,
                                               unsigned local, int lane) {
-    constexpr int VEC = DefaultVec<S>::value;
+    constexpr int VEC = StepVec<S>::value;
     Diag dg;
     const unsigned s = local + lane;
     const S* src = static_cast<const S*>(e.src);
@@ -850,6 +870,8 @@ __device__ __forceinline__ void group_segment(const GroupEntry& e, const Consts<
 
 template <typename S, bool SHIFT>
 __global__ void __launch_bounds__(256) group_step_kernel(const __grid_constant__ GroupArgs g) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     using T = typename Conv<S>::T;
     const int lane = threadIdx.x & 31;
     const unsigned stride = gridDim.x * blockDim.x;

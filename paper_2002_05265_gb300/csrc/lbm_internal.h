@@ -46,6 +46,9 @@ const void* batch_kernel_f32(int vec, int block);
 const void* batch_kernel_f16(int vec, int block);
 const void* batch_kernel_bf16(int vec, int block);
 
+// CTA size for a grid-stride kernel of so many threads: 256, or less where two CTAs per SM would not
+// be filled, down to a warp.
+int spread_block(long long threads);
 // Vector width (nodes per thread) of the step kernel for a storage type.
 int storage_vec(int storage);
 // Bytes per stored population.
