@@ -9,6 +9,14 @@
 // per-thread Householder reduction to upper Hessenberg form and the shifted QR iteration
 // (Francis / Wilkinson shift from the trailing 2 x 2 block, Givens rotations, deflation on
 // negligible subdiagonal entries), in FP64.
+//
+// The FP64 pipe bounds the solver: a scheduler takes 64 clocks for an FP64 instruction of a warp, so
+// one warp each keeps the pipe busy and what counts is the number of operations.  Only eigenvalues
+// are wanted, so rotations stay inside the active block; a rotation takes one reciprocal square root
+// instead of four hypot and four divisions; magnitudes in tests are |re| + |im|; the largest |lambda|
+// is found squared, with one logarithm at the end; the phases of E^D are products of two.  The
+// matrices live in shared memory, 16 bytes an entry and lane (the local arrays of before did not fit
+// the L1).  Measured, 16 flows x 64 x 64 wavenumbers of K: 7.7 -> 3.5 ms.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -32,134 +40,177 @@ __device__ __forceinline__ Cx operator*(Cx a, Cx b) {
 }
 __device__ __forceinline__ Cx operator*(double s, Cx a) { return Cx{s * a.re, s * a.im}; }
 __device__ __forceinline__ Cx conj(Cx a) { return Cx{a.re, -a.im}; }
-__device__ __forceinline__ double cabs(Cx a) { return hypot(a.re, a.im); }
-__device__ __forceinline__ Cx cdiv(Cx a, Cx b) {
-    const double d = b.re * b.re + b.im * b.im;
-    return Cx{(a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d};
-}
+__device__ __forceinline__ double norm2(Cx a) { return a.re * a.re + a.im * a.im; }
+__device__ __forceinline__ double abs1(Cx a) { return fabs(a.re) + fabs(a.im); }
 // principal square root
 __device__ __forceinline__ Cx csqrt(Cx a) {
-    const double r = cabs(a);
+    const double r = sqrt(norm2(a));
     if (r == 0.0) return cx(0.0);
-    const double t = sqrt(0.5 * (r + fabs(a.re)));
-    if (a.re >= 0.0) return Cx{t, a.im / (2.0 * t)};
-    return Cx{fabs(a.im) / (2.0 * t), a.im >= 0.0 ? t : -t};
+    const double t = sqrt(0.5 * (r + fabs(a.re))), q = a.im / (2.0 * t);
+    if (a.re >= 0.0) return Cx{t, q};
+    return Cx{fabs(q), a.im >= 0.0 ? t : -t};
 }
 
 constexpr int N = 9;
+constexpr int kEigLanes = 32;   // matrices of a CTA
 
-// Eigenvalues of the complex N x N matrix a (row-major, overwritten).  Returns the number of
-// QR sweeps, or -1 if an eigenvalue did not converge within the sweep limit.
-__device__ int eig9(Cx (&a)[N][N], Cx (&lam)[N]) {
-    // Householder reduction to upper Hessenberg form: for column c, zero a[c+2..][c]
-    for (int c = 0; c < N - 2; ++c) {
-        double alpha2 = 0.0;
-        for (int r = c + 1; r < N; ++r) alpha2 += a[r][c].re * a[r][c].re + a[r][c].im * a[r][c].im;
-        const double alpha = sqrt(alpha2);
-        if (alpha == 0.0) continue;
-        const Cx x0 = a[c + 1][c];
-        const double ax0 = cabs(x0);
-        const Cx ph = ax0 > 0.0 ? Cx{x0.re / ax0, x0.im / ax0} : cx(1.0);
-        // v = x + ph * alpha e_1, H = I - 2 v v^H / (v^H v)
-        Cx v[N];
-        for (int r = 0; r < N; ++r) v[r] = cx(0.0);
-        for (int r = c + 1; r < N; ++r) v[r] = a[r][c];
-        v[c + 1] = v[c + 1] + alpha * ph;
-        double vn = 0.0;
-        for (int r = c + 1; r < N; ++r) vn += v[r].re * v[r].re + v[r].im * v[r].im;
-        if (vn == 0.0) continue;
-        const double s = 2.0 / vn;
-        // a <- H a
-        for (int j = 0; j < N; ++j) {
-            Cx d = cx(0.0);
-            for (int r = c + 1; r < N; ++r) d = d + conj(v[r]) * a[r][j];
-            for (int r = c + 1; r < N; ++r) a[r][j] = a[r][j] - s * (v[r] * d);
-        }
-        // a <- a H
-        for (int i = 0; i < N; ++i) {
-            Cx d = cx(0.0);
-            for (int r = c + 1; r < N; ++r) d = d + a[i][r] * v[r];
-            for (int r = c + 1; r < N; ++r) a[i][r] = a[i][r] - s * (d * conj(v[r]));
-        }
-        for (int r = c + 2; r < N; ++r) a[r][c] = cx(0.0);
+// A lane's matrix in shared memory.
+struct Matrix {
+    double2* p;
+    __device__ __forceinline__ Cx get(int r, int c) const {
+        const double2 v = p[(r * N + c) * kEigLanes];
+        return Cx{v.x, v.y};
     }
+    __device__ __forceinline__ void set(int r, int c, Cx v) const { p[(r * N + c) * kEigLanes] = make_double2(v.re, v.im); }
+};
+
+// Column C of the Householder reduction to upper Hessenberg form: zeroes a[C + 2 ..][C].
+template <int C>
+__device__ __forceinline__ void hessenberg_column(const Matrix& a) {
+    constexpr int M = N - 1 - C;   // rows C + 1 .. N - 1
+    Cx v[M];
+    double alpha2 = 0.0;
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+        v[r] = a.get(C + 1 + r, C);
+        alpha2 += norm2(v[r]);
+    }
+    if (alpha2 == 0.0) return;
+    const double alpha = sqrt(alpha2), x2 = norm2(v[0]);
+    const double ix = x2 > 0.0 ? rsqrt(x2) : 0.0;
+    const Cx ph = x2 > 0.0 ? ix * v[0] : cx(1.0);
+    // v = x + ph alpha e_1, H = I - 2 v v^H / (v^H v), v^H v = 2 (alpha^2 + alpha |x_1|)
+    const double s = 1.0 / (alpha2 + alpha * (x2 * ix));
+    v[0] = v[0] + alpha * ph;
+    a.set(C + 1, C, -alpha * ph);
+#pragma unroll
+    for (int r = 1; r < M; ++r) a.set(C + 1 + r, C, cx(0.0));
+#pragma unroll 1
+    for (int j = C + 1; j < N; ++j) {   // a <- H a
+        Cx x[M], d = cx(0.0);
+#pragma unroll
+        for (int r = 0; r < M; ++r) {
+            x[r] = a.get(C + 1 + r, j);
+            d = d + conj(v[r]) * x[r];
+        }
+        d = s * d;
+#pragma unroll
+        for (int r = 0; r < M; ++r) a.set(C + 1 + r, j, x[r] - v[r] * d);
+    }
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {   // a <- a H
+        Cx x[M], d = cx(0.0);
+#pragma unroll
+        for (int r = 0; r < M; ++r) {
+            x[r] = a.get(i, C + 1 + r);
+            d = d + x[r] * v[r];
+        }
+        d = s * d;
+#pragma unroll
+        for (int r = 0; r < M; ++r) a.set(i, C + 1 + r, x[r] - d * conj(v[r]));
+    }
+}
+
+// Eigenvalues of the complex N x N matrix a (overwritten), each handed to `found` with its index.
+// Returns the number of QR sweeps, or -1 if an eigenvalue did not converge within the sweep limit.
+template <typename Found>
+__device__ int eig9(const Matrix& a, Found found) {
+    hessenberg_column<0>(a);
+    hessenberg_column<1>(a);
+    hessenberg_column<2>(a);
+    hessenberg_column<3>(a);
+    hessenberg_column<4>(a);
+    hessenberg_column<5>(a);
+    hessenberg_column<6>(a);
     // shifted QR on the active block [lo, hi]; a subdiagonal entry is negligible against its
     // two diagonal neighbours, or against the matrix norm when both are tiny (zero eigenvalues:
     // with omega_3 = omega_4 = 1 the collision removes whole moments)
     double anorm = 0.0;
+#pragma unroll 1
     for (int i = 0; i < N; ++i)
-        for (int j = 0; j < N; ++j) anorm += a[i][j].re * a[i][j].re + a[i][j].im * a[i][j].im;
+#pragma unroll 1
+        for (int j = i > 0 ? i - 1 : 0; j < N; ++j) anorm += norm2(a.get(i, j));
     anorm = sqrt(anorm);
     int hi = N - 1, sweeps = 0;
     while (hi >= 0) {
-        if (hi == 0) {
-            lam[0] = a[0][0];
-            break;
-        }
         // deflation: find the start of the unreduced block ending at hi
         int lo = hi;
+        double below = abs1(a.get(hi, hi));
         while (lo > 0) {
-            const double sc = cabs(a[lo][lo]) + cabs(a[lo - 1][lo - 1]);
-            if (cabs(a[lo][lo - 1]) <= 1e-15 * fmax(sc, 1e-3 * anorm)) {
-                a[lo][lo - 1] = cx(0.0);
+            const double above = abs1(a.get(lo - 1, lo - 1));
+            if (abs1(a.get(lo, lo - 1)) <= 1e-15 * fmax(below + above, 1e-3 * anorm)) {
+                a.set(lo, lo - 1, cx(0.0));
                 break;
             }
+            below = above;
             --lo;
         }
         if (lo == hi) {
-            lam[hi] = a[hi][hi];
+            found(hi, a.get(hi, hi));
             --hi;
             continue;
         }
         if (++sweeps > 60 * N) return -1;
         // Wilkinson shift: eigenvalue of the trailing 2 x 2 block closest to a[hi][hi]
-        const Cx p = a[hi - 1][hi - 1], q = a[hi - 1][hi], r = a[hi][hi - 1], t = a[hi][hi];
-        const Cx half_tr = 0.5 * (p + t);
-        const Cx disc = csqrt(0.25 * ((p - t) * (p - t)) + q * r);
-        const Cx e1 = half_tr + disc, e2 = half_tr - disc;
-        Cx mu = cabs(e1 - t) < cabs(e2 - t) ? e1 : e2;
+        const Cx p = a.get(hi - 1, hi - 1), q = a.get(hi - 1, hi), r = a.get(hi, hi - 1), t = a.get(hi, hi);
+        const Cx half_diff = 0.5 * (p - t), disc = csqrt(half_diff * half_diff + q * r);
+        // (e - t) = (p - t) / 2 +- disc, the smaller of the two
+        const Cx e1 = half_diff + disc, e2 = half_diff - disc;
+        Cx mu = t + (norm2(e1) < norm2(e2) ? e1 : e2);
         if (sweeps % 11 == 10) {   // exceptional shift, rotating in the complex plane
-            const double e = 0.75 * (cabs(a[hi][hi - 1]) + cabs(a[hi - 1][hi - 2 >= 0 ? hi - 2 : 0]));
+            const double e = 0.75 * (abs1(r) + abs1(a.get(hi - 1, hi - 2 >= 0 ? hi - 2 : 0)));
             double sn, cn;
             sincos(0.7 * sweeps, &sn, &cn);
-            mu = a[hi][hi] + Cx{e * cn, e * sn};
+            mu = t + Cx{e * cn, e * sn};
         }
-        // QR step on a[lo..hi] - mu I with Givens rotations, then RQ + mu I
-        Cx cs[N];
-        double cc[N];
-        for (int k = lo; k <= hi; ++k) a[k][k] = a[k][k] - mu;
-        for (int k = lo; k < hi; ++k) {
-            const Cx x = a[k][k], y = a[k + 1][k];
-            const double nrm = hypot(cabs(x), cabs(y));
-            double c;
-            Cx sgn;
-            if (nrm == 0.0) {
-                c = 1.0;
-                sgn = cx(0.0);
-            } else {
-                c = cabs(x) / nrm;
-                const Cx ph = cabs(x) > 0.0 ? Cx{x.re / cabs(x), x.im / cabs(x)} : cx(1.0);
-                sgn = (1.0 / nrm) * (ph * conj(y));   // s such that [c s; -conj(s) c] [x; y] = [., 0]
+        // QR step on a[lo..hi] - mu I with Givens rotations, then RQ + mu I.  Rotation k takes rows
+        // k, k + 1; the columns k - 1, k take rotation k - 1 right after it, when their rows up to k
+        // are those of R.
+        double c0 = 1.0;
+        Cx s0 = cx(0.0);
+        a.set(lo, lo, a.get(lo, lo) - mu);
+#pragma unroll 1
+        for (int k = lo; k <= hi; ++k) {
+            double c = 1.0;
+            Cx sn = cx(0.0);
+            if (k < hi) {
+                a.set(k + 1, k + 1, a.get(k + 1, k + 1) - mu);
+                // c = |x| / n, s = (x / |x|) conj(y) / n, n^2 = |x|^2 + |y|^2:
+                // [c s; -conj(s) c] [x; y] = [., 0]
+                const Cx x = a.get(k, k), y = a.get(k + 1, k);
+                const double x2 = norm2(x), n2 = x2 + norm2(y);
+                if (x2 * n2 > 1e-290) {
+                    const double d = rsqrt(x2 * n2);
+                    c = x2 * d;
+                    sn = d * (x * conj(y));
+                    a.set(k, k, (n2 * d) * x);
+                } else if (n2 > 0.0) {   // x vanishes (to 1e-75 at least): swap the rows
+                    const double d = rsqrt(n2);
+                    c = 0.0;
+                    sn = d * conj(y);
+                    a.set(k, k, cx(n2 * d));
+                }
+                a.set(k + 1, k, cx(0.0));
+#pragma unroll 1
+                for (int j = k + 1; j <= hi; ++j) {
+                    const Cx u = a.get(k, j), w = a.get(k + 1, j);
+                    a.set(k, j, c * u + sn * w);
+                    a.set(k + 1, j, c * w - conj(sn) * u);
+                }
             }
-            cc[k] = c;
-            cs[k] = sgn;
-            for (int j = k; j < N; ++j) {
-                const Cx u = a[k][j], w = a[k + 1][j];
-                a[k][j] = c * u + sgn * w;
-                a[k + 1][j] = c * w - conj(sgn) * u;
+            if (k > lo) {
+#pragma unroll 1
+                for (int i = lo; i <= k; ++i) {
+                    const Cx u = a.get(i, k - 1), w = a.get(i, k);
+                    a.set(i, k - 1, c0 * u + conj(s0) * w);
+                    a.set(i, k, c0 * w - s0 * u);
+                }
+                a.set(k - 1, k - 1, a.get(k - 1, k - 1) + mu);
             }
+            c0 = c;
+            s0 = sn;
         }
-        for (int k = lo; k < hi; ++k) {
-            const double c = cc[k];
-            const Cx sgn = cs[k];
-            const int top = (k + 2 <= hi) ? k + 2 : hi;
-            for (int i = 0; i <= top; ++i) {
-                const Cx u = a[i][k], w = a[i][k + 1];
-                a[i][k] = c * u + conj(sgn) * w;
-                a[i][k + 1] = c * w - sgn * u;
-            }
-        }
-        for (int k = lo; k <= hi; ++k) a[k][k] = a[k][k] + mu;
+        a.set(hi, hi, a.get(hi, hi) + mu);
     }
     return sweeps;
 }
@@ -219,36 +270,43 @@ __global__ void lsa_jacobian_bgk_kernel(const double* __restrict__ flows, int nf
 }
 
 // growth[f * nk + k] = max_j ln |lambda_j(E^D(k) G_f)|; eig (optional) the eigenvalues.
-__global__ void lsa_growth_kernel(const double* __restrict__ G, int nflows, const double* __restrict__ kvec, int nk,
-                                  double* __restrict__ growth, double* __restrict__ eig, int* __restrict__ failed) {
-    const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kEigLanes) lsa_growth_kernel(const double* __restrict__ G, int nflows,
+                                                               const double* __restrict__ kvec, int nk,
+                                                               double* __restrict__ growth, double* __restrict__ eig,
+                                                               int* __restrict__ failed) {
+    __shared__ double2 sm[N * N * kEigLanes];
+    const long long id = blockIdx.x * (long long)kEigLanes + threadIdx.x;
     if (id >= (long long)nflows * nk) return;
     const int f = (int)(id / nk), k = (int)(id - (long long)f * nk);
-    const double kx = kvec[2 * k], ky = kvec[2 * k + 1];
-    Cx a[N][N], lam[N];
+    const Matrix a{sm + threadIdx.x};
+    // exp(-i k_x), exp(-i k_y) and their products
+    Cx ex[3], ey[3];   // index: velocity component + 1
+    double sn, cn;
+    sincos(kvec[2 * k], &sn, &cn);
+    ex[0] = Cx{cn, sn}; ex[1] = cx(1.0); ex[2] = Cx{cn, -sn};
+    sincos(kvec[2 * k + 1], &sn, &cn);
+    ey[0] = Cx{cn, sn}; ey[1] = cx(1.0); ey[2] = Cx{cn, -sn};
+#pragma unroll
     for (int i = 0; i < N; ++i) {
-        double sn, cn;
-        sincos(-(ex_of(i) * kx + ey_of(i) * ky), &sn, &cn);
-        for (int j = 0; j < N; ++j) {
-            const double gij = G[(long long)f * 81 + i * 9 + j];
-            a[i][j] = Cx{cn * gij, sn * gij};
-        }
+        const Cx e = ex_of(i) == 0 ? ey[ey_of(i) + 1] : (ey_of(i) == 0 ? ex[ex_of(i) + 1] : ex[ex_of(i) + 1] * ey[ey_of(i) + 1]);
+#pragma unroll
+        for (int j = 0; j < N; ++j) a.set(i, j, G[(long long)f * 81 + i * 9 + j] * e);
     }
-    if (eig9(a, lam) < 0) {
+    double best = -1.0;
+    const int sweeps = eig9(a, [&](int i, Cx lam) {
+        const double m = norm2(lam);
+        best = m > best ? m : best;
+        if (eig) {
+            eig[id * 18 + 2 * i] = lam.re;
+            eig[id * 18 + 2 * i + 1] = lam.im;
+        }
+    });
+    if (sweeps < 0) {
         atomicExch(failed, 1);
         growth[id] = nan("");
         return;
     }
-    double best = -1e300;
-    for (int i = 0; i < N; ++i) {
-        const double m = log(cabs(lam[i]));
-        best = m > best ? m : best;
-        if (eig) {
-            eig[id * 18 + 2 * i] = lam[i].re;
-            eig[id * 18 + 2 * i + 1] = lam[i].im;
-        }
-    }
-    growth[id] = best;
+    growth[id] = best > 0.0 ? 0.5 * log(best) : -1e300;
 }
 
 template <int MODEL>
@@ -318,7 +376,7 @@ extern "C" int lbm_lsa_growth(int model, lbm_rates rates, int eq_order, const do
     }
     if (e == cudaSuccess) {
         const long long n = (long long)nflows * nk;
-        lsa_growth_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(G, nflows, k, nk, growth, eig, failed);
+        lsa_growth_kernel<<<(unsigned)((n + kEigLanes - 1) / kEigLanes), kEigLanes, 0, s>>>(G, nflows, k, nk, growth, eig, failed);
         e = cudaGetLastError();
     }
     int h_failed = 0;
