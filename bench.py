@@ -4,8 +4,9 @@ Workload (one benchmark step): the periodic double shear layer on 1024 x 1024 la
 (tanh width L/80, Ma = 0.1, transverse perturbation 0.05, nu = 1e-5), one lattice per
 collision model (BGK, RM, HM, CM, CHM, K, PR, RR; FP32 shifted storage, FP32 collision),
 each initialised at equilibrium, advanced 20000 time steps with the FP64 blow-up check every
-100 steps, and reduced to its moments.  The eight lattices advance together, one time step
-of each in turn, so the 604 MB working set streams from HBM (larger than the 126 MB L2).
+100 steps, and reduced to its moments.  The eight lattices advance together, a few time steps of
+all of them per launch, so the 604 MB working set streams from HBM (larger than the 126 MB L2)
+once per launch.
 
 Metric: lattice updates per second (GLUPS) over all lattices; `e2e` repeats the step through
 the same C calls with pinned host buffers (host->device copy of rho, u and device->host copy
@@ -1051,26 +1052,39 @@ def main():
     lu_per_step = len(MODELS) * L * L * S
     value = world * lu_per_step * args.steps / (ms / 1e3) / 1e9
 
-    # dominant kernel: the multi-lattice step kernel (one launch advances the 8 lattices one
-    # time step); average launch duration from the CUDA events around every graph replay of
-    # the timed region (the graphs contain only step launches)
+    # dominant kernel: the multi-lattice step kernel (one launch advances the 8 lattices
+    # `fused` time steps and moves their populations once); average launch duration from the
+    # CUDA events around every graph replay of the timed region (the graphs contain only step
+    # launches)
     peak, peak_kind = measured_peaks()
     avg_launch_s = replay_ms / 1e3 / kernel_launches
-    bytes_per_launch = BYTES_PER_LU["f32"] * L * L * lattice_steps / kernel_launches
+    fused = lattice_steps / kernel_launches / len(MODELS)
+    desc = lbm.lbm_group_describe(group)
+    # every choice left to the library: fused launches (lbm_group_describe tells the one-step form)
+    marched = (fused > 1 and args.path == "auto" and args.form == "auto" and args.order == "auto" and
+               not args.stages and not args.launch_steps)
+    # launches of the copy-engine kernel with several steps move the populations at every step
+    bytes_per_launch = BYTES_PER_LU["f32"] * L * L * len(MODELS) * (1 if marched else fused)
     achieved = bytes_per_launch / avg_launch_s / 1e9
     form = form_name(lbm, group)
-    bulk = form != "register-staged"
-    # the committed ncu traffic records: the wide form (the default here) and the
-    # register-staged group kernel
-    traffic = ncu_traffic("f32_tile_8x1024") if form == "wide" else (
-        ncu_traffic("f32_group_8x1024") if not bulk else None)
-    kname = (f"lbm::tile_step_kernel<float> (cp.async.bulk ring, {form} form)" if bulk
-             else "lbm::group_step_kernel<float> (register-staged)")
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": traffic, "peak_source": peak_kind, "launch_us": avg_launch_s * 1e6,
-                "bytes_per_launch": bytes_per_launch,
-                "kernel": kname + f": one launch = {lattice_steps // kernel_launches // len(MODELS)} time step(s) "
-                          "of the 8 lattices, 72 B per lattice update"}
+    bulk = desc["family"] == lbm.LBM_PATH_BULK
+    # the committed ncu traffic records
+    traffic = ncu_traffic("f32_march_8x1024" if marched else
+                          ("f32_tile_8x1024" if form == "wide" else "f32_group_8x1024"))
+    if marched:
+        kname = "lbm::march_kernel<float> (time-fused)"
+    elif bulk:
+        kname = f"lbm::tile_step_kernel<float> (cp.async.bulk ring, {form} form)"
+    else:
+        kname = "lbm::group_step_kernel<float> (register-staged)"
+    roofline = {"bound": "fp32" if marched else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak, "traffic": traffic, "peak_source": peak_kind,
+                "launch_us": avg_launch_s * 1e6, "bytes_per_launch": bytes_per_launch, "steps_per_launch": fused,
+                "one_step_floor_us": BYTES_PER_LU["f32"] * L * L * len(MODELS) / peak / 1e3,
+                "step_us": avg_launch_s * 1e6 / fused,
+                "kernel": kname + f": one launch = {fused:g} time step(s) of the 8 lattices"
+                          + (", their populations read and written once (72 B per node)" if marched
+                             else ", 72 B per lattice update")}
 
     # step-kernel launches counted by the group's replay timing, plus one reduction launch per
     # check of the eight lattices (they fall due together and share a launch; each lattice's
