@@ -95,9 +95,11 @@ __global__ void scatter_kernel(S* buf, FieldArgs a, const double* __restrict__ f
 // that pipe bounded the kernel (37.4 ms at 16384^2, 16 GB to move).  So FP32 values are widened
 // with integer operations; their sums are taken exactly in FP32 by error-free two-sums (Knuth), two
 // nodes per instruction, and only closed in FP64; u takes one reciprocal for both components by a
-// Newton step from the FP32 one and closes each quotient with its remainder (Markstein).  That
+// Newton step from the FP32 one and closes each quotient with its remainder (Markstein).  The
+// start is the reciprocal of the closed density's upper bits, so that it is good to 2^-22 at any
+// density; a node whose density or sums leave the range in which this holds is summed plainly.  That
 // leaves 12 FP64 operations a node: 37.4 -> 10.5 ms at 16384^2, 155 -> 55 us at 1024^2; errors as
-// before (rho 1.7e-16, u 1.7e-17 at most, against long double).
+// before (rho 1.7e-16, u 1.7e-17 at most, against long double, at densities near 1).
 
 // the double of a float's value
 __device__ __forceinline__ double widen(float v) {
@@ -106,6 +108,14 @@ __device__ __forceinline__ double widen(float v) {
     const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
     return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
+
+// The float of a double's upper 24 bits, by integer operations; false unless 2^-50 <= |v| < 2^50.
+__device__ __forceinline__ bool narrow(double v, float& f) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), m = hi & 0x7fffffffu;
+    f = __uint_as_float((hi & 0x80000000u) | ((m - 0x38000000u) << 3) | ((uint32_t)__double2loint(v) >> 29));
+    return (m >> 20) - 973u < 100u;
+}
+__device__ __forceinline__ bool finite(double v) { return ((uint32_t)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u; }
 
 // s + e = a + b exactly
 __device__ __forceinline__ void two_sum(F2 a, F2 b, F2& s, F2& e) {
@@ -237,33 +247,42 @@ __global__ void __launch_bounds__(kBlock) gather_kernel(const S* buf, FieldArgs 
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             if (j >= nvalid) continue;
-            const float drf = j ? f2_hi(dr.hi) : f2_lo(dr.hi), jxf = j ? f2_hi(jx.hi) : f2_lo(jx.hi);
-            const float jyf = j ? f2_hi(jy.hi) : f2_lo(jy.hi);
-            const float rf = (float)a.rho0 + drf;
-            // the exact sums and the quotients below want ordinary values; the others go the plain way
-            if (!(fabsf(drf) < 1e15f && fabsf(rf) > 1e-15f && fabsf(jxf) < 1e15f && fabsf(jyf) < 1e15f)) {
+            const double r = a.rho0 + dr.value(j);
+            float rf;
+            bool ordinary = narrow(r, rf);
+            double u[2] = {0.0, 0.0}, p2[3] = {0.0, 0.0, 0.0};
+            if (o.ux || o.uy) {
+                const double r0 = widen(rcp_approx(rf)), r1 = fma(r0, fma(-r, r0, 1.0), r0);
+                if (o.ux) {
+                    const double q = shifted ? fma(a.rho0, a.urx, jx.value(j)) : jx.value(j), v = q * r1;
+                    u[0] = fma(fma(-r, v, q), r1, v);
+                }
+                if (o.uy) {
+                    const double q = shifted ? fma(a.rho0, a.ury, jy.value(j)) : jy.value(j), v = q * r1;
+                    u[1] = fma(fma(-r, v, q), r1, v);
+                }
+                ordinary = ordinary && finite(u[0]) && finite(u[1]);
+            }
+            if (o.second()) {
+                p2[0] = fma(a.rho0, c.second[0], sxx.value(j));
+                p2[1] = fma(c.second[1], a.ury, sxy.value(j));
+                p2[2] = fma(a.rho0, c.second[2], syy.value(j));
+                ordinary = ordinary && finite(p2[0]) && finite(p2[1]) && finite(p2[2]);
+            }
+            // a density far from 1 or a sum beyond the FP32 range: the plain way
+            if (!ordinary) {
                 double d[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) d[i] = (double)g[i][j];
                 moments_plain<true>(d, a, o, k + j);
                 continue;
             }
-            const double r = a.rho0 + dr.value(j);
             if (o.rho) o.rho[k + j] = r;
-            if (o.ux || o.uy) {
-                const double r0 = widen(rcp_approx(rf)), r1 = fma(r0, fma(-r, r0, 1.0), r0);
-                if (o.ux) {
-                    const double q = shifted ? fma(a.rho0, a.urx, jx.value(j)) : jx.value(j), u = q * r1;
-                    o.ux[k + j] = fma(fma(-r, u, q), r1, u);
-                }
-                if (o.uy) {
-                    const double q = shifted ? fma(a.rho0, a.ury, jy.value(j)) : jy.value(j), u = q * r1;
-                    o.uy[k + j] = fma(fma(-r, u, q), r1, u);
-                }
-            }
-            if (o.pxx) o.pxx[k + j] = fma(a.rho0, c.second[0], sxx.value(j));
-            if (o.pxy) o.pxy[k + j] = fma(c.second[1], a.ury, sxy.value(j));
-            if (o.pyy) o.pyy[k + j] = fma(a.rho0, c.second[2], syy.value(j));
+            if (o.ux) o.ux[k + j] = u[0];
+            if (o.uy) o.uy[k + j] = u[1];
+            if (o.pxx) o.pxx[k + j] = p2[0];
+            if (o.pxy) o.pxy[k + j] = p2[1];
+            if (o.pyy) o.pyy[k + j] = p2[2];
         }
     }
 }
