@@ -4,9 +4,9 @@
 //
 // GB300 has 2 FP64 lanes per SM and clock, conversions included; nine populations are about 150
 // FP64 operations, and that pipe bounded the initialisation (36.6 ms at 16384^2, 16 GB to move).  So
-// g is evaluated in pairs of floats (about 2^-44 of its terms) and rounded from there when every
-// value within the error bound rounds alike, which decides all but some 10^-4 of the populations
-// (rounding test: Ziv 1991); the others take the FP64 expressions.
+// g is evaluated in pairs of floats (to 2^-40 of the sum of its terms' sizes, see equilibrium_node)
+// and rounded from there when every value within that bound rounds alike (rounding test: Ziv 1991);
+// the few others take the FP64 expressions.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -28,8 +28,8 @@ __device__ __forceinline__ Wide wide_add(Wide a, Wide b) {   // two-sum (Knuth) 
 }
 __device__ __forceinline__ Wide wide_scale(Wide a, float c) { return Wide{a.h * c, a.l * c}; }   // c = +-2^k
 // x as the float of its upper 24 bits and the float nearest to the rest, by integer operations;
-// false unless x is zero or 2^-60 <= |x| < 2^60.
-__device__ __forceinline__ bool wide_split(double x, Wide& w) {
+// false unless x is zero or 2^LO <= |x| < 2^HI.
+template <int LO, int HI> __device__ __forceinline__ bool wide_split(double x, Wide& w) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
     const uint32_t sign = hi & 0x80000000u, m = hi & 0x7fffffffu, e = m >> 20;
     if ((m | lo) == 0u) {
@@ -40,7 +40,7 @@ __device__ __forceinline__ bool wide_split(double x, Wide& w) {
     // the lower 29 bits, in units of 2^(e - 1023 - 52)
     const float unit = __uint_as_float(sign | ((e - (1023u + 52u - 127u)) << 23));
     w.l = (float)(lo & 0x1fffffffu) * unit;
-    return e - 963u < 120u;
+    return e - (uint32_t)(1023 + LO) < (uint32_t)(HI - LO);
 }
 
 // Rounds h + l +- err to the storage type; false if that interval holds values that round apart.
@@ -71,9 +71,10 @@ __device__ __forceinline__ double equilibrium_plain(int i, double r, double vx, 
     return Px * Py * (r - rho0) + r * (Px * Dy + Dx * (Py + Dy));
 }
 
-// The shift's factors P_0, P_+, P_- per axis as pairs of floats.
+// The shift's factors P_0, P_+, P_- per axis as pairs of floats, and |P_0|, the larger of |P_+-|.
 struct EquilibriumConsts {
     float2 px[3], py[3];
+    float ax[2], ay[2];
 };
 __host__ __device__ inline EquilibriumConsts equilibrium_consts(double urx, double ury) {
     EquilibriumConsts c;
@@ -82,6 +83,10 @@ __host__ __device__ inline EquilibriumConsts equilibrium_consts(double urx, doub
         const double x = phi1d(s, urx), y = phi1d(s, ury);
         c.px[k] = make_float2((float)x, (float)(x - (double)(float)x));
         c.py[k] = make_float2((float)y, (float)(y - (double)(float)y));
+        // (2^-12 at least: P itself carries 2^-53, whatever is left of it next to its zero)
+        const float ax = fmaxf(fabsf(c.px[k].x), 0x1p-12f), ay = fmaxf(fabsf(c.py[k].x), 0x1p-12f);
+        c.ax[k != 0] = k == 2 ? fmaxf(c.ax[1], ax) : ax;
+        c.ay[k != 0] = k == 2 ? fmaxf(c.ay[1], ay) : ay;
     }
     return c;
 }
@@ -93,13 +98,15 @@ __device__ __forceinline__ void equilibrium_node(double r, double vx, double vy,
 #pragma unroll
         for (int i = 0; i < 9; ++i) g[i] = equilibrium_plain(i, r, vx, vy, rho0, urx, ury);
     } else {
+        // ranges in which no product below leaves the FP32 range (see the error bound)
         Wide R, dr, dx, dy, sx, sy;
-        bool sure = wide_split(r, R) && wide_split(r - rho0, dr) && wide_split(vx - urx, dx) && wide_split(vy - ury, dy);
+        bool sure = wide_split<-20, 20>(r, R) && wide_split<-60, 20>(r - rho0, dr) &&
+                    wide_split<-60, 2>(vx - urx, dx) && wide_split<-60, 2>(vy - ury, dy);
         if (urx == 0.0 && ury == 0.0) {
             sx = dx;
             sy = dy;
         } else {
-            sure = sure && wide_split(vx + urx, sx) && wide_split(vy + ury, sy);
+            sure = sure && wide_split<-60, 2>(vx + urx, sx) && wide_split<-60, 2>(vy + ury, sy);
         }
         // order 0, +, -: D_0 = -d s, D_+- = (d s +- d) / 2
         const Wide X = wide_mul(dx, sx), Y = wide_mul(dy, sy);
@@ -107,12 +114,28 @@ __device__ __forceinline__ void equilibrium_node(double r, double vx, double vy,
                             wide_scale(wide_add(X, wide_scale(dx, -1.0f)), 0.5f)};
         const Wide Dy[3] = {wide_scale(Y, -1.0f), wide_scale(wide_add(Y, dy), 0.5f),
                             wide_scale(wide_add(Y, wide_scale(dy, -1.0f)), 0.5f)};
-        // error bound: a product of three wide factors is off by less than 2^-43.4 of it (2^-45 for
-        // each product, the sums less), and for |u + u_ref| < 1 a population's terms are together
-        // less than this size (largest error found over 2 x 10^7 random nodes: 2^-44.6 of it)
-        const float size = fabsf(dr.h) + fabsf(R.h) * (fabsf(dx.h) + fabsf(dy.h));
-        const float err = size * 1.1368683772161603e-13f;   // 2^-43
-        sure = sure && fabsf(sx.h) < 1.0f && fabsf(sy.h) < 1.0f;
+        // Error bound, in u = 2^-24.  Let M be the sum of the sizes of the terms a value is made of.  A
+        // split is off by 2 u^2 M with a low part of 2 u M, P by u^2 M and u M; a wide product of (e, l)
+        // and (e', l') by e + e' + l + 2 l' + 2 + l l' with a low part of l + l' + 1; a wide sum by
+        // max(e) + 2 max(l) + 1 with max(l) + 1.  So d s is off by 16 (low part 5), D by 27 (6), rho D
+        // by 57 (9), H and K by 76 (10), P H by 110 (12), D K by 191 (17) and g by 226 (18).  The
+        // rounding of l +- err adds 18, FP64's own less than 1: 2^8 u^2 = 2^-40.  M = |P| (|P'| |dr| +
+        // |rho| |D'|) + |D| |rho| (|P'| + |D'|) with |d s| and (|d s| + |d|) / 2 for |D_0| and |D_+-|.
+        // Underflow: at most 40 operations lose 2^-150 each, times at most 2^20 2^6 after it; below
+        // M = 2^-110 nothing but zero is sure.  (With one bound for all nine, |dr| + |rho| (|d_x| + |d_y|)
+        // times 2^-43, M was larger by up to 2.4 for |u_ref| near 1.)
+        const float mX = fabsf(X.h), mY = fabsf(Y.h), mR = fabsf(R.h), mr = fabsf(dr.h);
+        const float mDx[2] = {mX, 0.5f * (mX + fabsf(dx.h))}, mDy[2] = {mY, 0.5f * (mY + fabsf(dy.h))};
+        float err[2][2];   // [xi_x != 0][xi_y != 0]
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const float mH = fmaf(c.ay[b], mr, mR * mDy[b]), mK = mR * (c.ay[b] + mDy[b]);
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const float M = fmaf(c.ax[a], mH, mDx[a] * mK);
+                err[a][b] = fmaf(M, 0x1p-40f, fminf(M, 0x1p-110f));
+            }
+        }
         unsigned open = sure ? 0u : 0x1ffu;   // populations that the bound leaves open
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
@@ -126,7 +149,7 @@ __device__ __forceinline__ void equilibrium_node(double r, double vx, double vy,
                 const Wide Px{c.px[a].x, c.px[a].y};
                 const Wide v = wide_add(wide_mul(Px, H), wide_mul(Dx[a], K));
                 S out;
-                const bool known = round_sure(v.h, v.l, err, out);
+                const bool known = round_sure(v.h, v.l, err[a != 0][b != 0], out);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
                     if (ex_of(i) != ex || ey_of(i) != ey) continue;

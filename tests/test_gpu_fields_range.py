@@ -85,3 +85,38 @@ def test_moments_at_any_reference_density(L, storage, rho0):
                                 (rho0, 1.0, 1.0, rho0, rho0, rho0)):
         off = np.abs(got / scale - want)
         assert float(np.max(off)) <= 2e-15, float(np.max(off))
+
+
+def _phi(s, u):
+    return np.longdouble(2) / 3 - u * u if s == 0 else (u * u + s * u + np.longdouble(1) / 3) / 2
+
+
+@pytest.mark.parametrize("storage,precision", [("f32", 24), ("f16", 11), ("bf16", 8)])
+@pytest.mark.parametrize("uref", [(0.0, 0.0), (0.9, 0.9), (-0.99, 0.3), (0.8164965, -0.8164966)])
+def test_equilibrium_far_from_the_reference_velocity(L, storage, precision, uref):
+    """2^20 nodes with |u| up to 1.9 about reference velocities up to 0.99: every stored g = f^eq - s
+    lies within half a unit in the last place of its exact value; 2^-49 allowed for its FP64
+    evaluation, terms of size up to 8 in FP64 (2^-52 of them), and for reading f = g + s back."""
+    n = 1024
+    g = np.random.Generator(np.random.Philox(8))
+    rho = 1.0 + 0.2 * g.uniform(-1, 1, (n, n))
+    ux, uy = (-r + g.uniform(-1, 1, (n, n)) if r else g.uniform(-1, 1, (n, n)) for r in uref)
+    lat = L.Lattice(n, n, "chm", (1.9, 1.2, 0.9), storage=L.STORAGES[storage])
+    if uref != (0.0, 0.0):
+        lat.set_shift_velocity(*uref)
+    lat.init_equilibrium(*[torch.from_numpy(v).cuda() for v in (rho, ux, uy)])
+    f = torch.empty((9, n, n), dtype=torch.float64, device="cuda")
+    lat.get_populations(f)
+    lat.close()
+    f = f.cpu().numpy()
+    R, X, Y = (v.astype(np.longdouble) for v in (rho, ux, uy))
+    ur = [np.longdouble(v) for v in uref]
+    for i in range(9):
+        s = _phi(EX[i], ur[0]) * _phi(EY[i], ur[1])
+        want = R * _phi(EX[i], X) * _phi(EY[i], Y) - s
+        off = np.abs(f[i] - s - want).astype(np.float64)
+        half = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(want).astype(np.float64), 1e-300))) - precision)
+        if storage == "f16":
+            half = np.maximum(half, 2.0 ** -25)   # subnormal halves
+        bad = off > half + 2.0 ** -49
+        assert not bad.any(), (i, int(bad.sum()), float(np.max((off - half)[bad])))
