@@ -146,71 +146,94 @@ struct ExactSum {
 
 struct MomentOut {
     double *rho, *ux, *uy, *pxx, *pxy, *pyy;
-    __device__ __forceinline__ bool any() const { return rho || ux || uy || pxx || pxy || pyy; }
+    __host__ __device__ __forceinline__ bool any() const { return rho || ux || uy || pxx || pxy || pyy; }
     __device__ __forceinline__ bool second() const { return pxx || pxy || pyy; }
 };
 
-// Moments of one node from its populations, one FP64 sum after another: every storage type's for a
-// node with a non-finite or extreme value, FP64 storage's always (there without the zero terms,
-// which change nothing where the density is finite).
-template <bool ZEROS>
+// The moments asked for, from the sums of one node's populations.
+__device__ __forceinline__ void moments_close(double dr, double jx, double jy, double sxx, double sxy, double syy,
+                                              const FieldArgs& a, const MomentOut& o, long long k) {
+    // moments of the shift: sum s = rho0, sum xi s = rho0 u_ref,
+    // sum xi_a xi_b s = rho0 (u_ref,a u_ref,b + c_s^2 delta_ab)
+    const double r = a.rho0 + dr;
+    if (o.rho) o.rho[k] = r;
+    if (o.ux) o.ux[k] = (jx + a.rho0 * a.urx) / r;
+    if (o.uy) o.uy[k] = (jy + a.rho0 * a.ury) / r;
+    if (o.pxx) o.pxx[k] = sxx + a.rho0 * (a.urx * a.urx + 1.0 / 3.0);
+    if (o.pxy) o.pxy[k] = sxy + a.rho0 * a.urx * a.ury;
+    if (o.pyy) o.pyy[k] = syy + a.rho0 * (a.ury * a.ury + 1.0 / 3.0);
+}
+// A node with a non-finite or extreme value: one FP64 sum over all nine populations after another
+// (a zero times an infinity shows).
 __device__ __forceinline__ void moments_plain(const double (&g)[9], const FieldArgs& a, const MomentOut& o, long long k) {
     double dr = 0, jx = 0, jy = 0, sxx = 0, sxy = 0, syy = 0;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int sx = ex_of(i), sy = ey_of(i);
-        dr += g[i];
-        if (ZEROS || sx) jx += sx * g[i];
-        if (ZEROS || sy) jy += sy * g[i];
-        if (ZEROS || sx) sxx += sx * sx * g[i];
-        if (ZEROS || sx * sy) sxy += sx * sy * g[i];
-        if (ZEROS || sy) syy += sy * sy * g[i];
+        dr += g[i]; jx += sx * g[i]; jy += sy * g[i];
+        sxx += sx * sx * g[i]; sxy += sx * sy * g[i]; syy += sy * sy * g[i];
     }
-    // moments of the shift: sum s = rho0, sum xi s = rho0 u_ref,
-    // sum xi_a xi_b s = rho0 (u_ref,a u_ref,b + c_s^2 delta_ab)
-    const double r = a.rho0 + dr;
-    jx += a.rho0 * a.urx;
-    jy += a.rho0 * a.ury;
-    if (o.rho) o.rho[k] = r;
-    if (o.ux) o.ux[k] = jx / r;
-    if (o.uy) o.uy[k] = jy / r;
-    if (o.pxx) o.pxx[k] = sxx + a.rho0 * (a.urx * a.urx + 1.0 / 3.0);
-    if (o.pxy) o.pxy[k] = sxy + a.rho0 * a.urx * a.ury;
-    if (o.pyy) o.pyy[k] = syy + a.rho0 * (a.ury * a.ury + 1.0 / 3.0);
+    moments_close(dr, jx, jy, sxx, sxy, syy, a, o, k);
 }
 
-// FP64 storage: one node per thread.
-__global__ void gather_kernel_f64(const double* buf, FieldArgs a, double* f, MomentOut o) {
-    if (a.which && *a.which) buf += a.other;
-    const long long n = (long long)a.nx * a.ny;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(k / a.nx), x = (int)(k - (long long)y * a.nx);
-        double g[9], dr = 0.0;
+// FP64 storage: one node per thread; the FP64 pipe bounds it, so only the sums that are asked for, and
+// without their zero terms, which change nothing where the density is finite.
+__global__ void __launch_bounds__(kBlock) moments_kernel_f64(const double* buf, FieldArgs a, MomentOut o) {
+    const unsigned n = (unsigned)a.nx * (unsigned)a.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int y = (int)(k / (unsigned)a.nx), x = (int)(k - (unsigned)y * (unsigned)a.nx);
+        double g[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            g[i] = buf[src_offset(i, x, y, a)];
-            dr += g[i];
-        }
-        if (f) {
+        for (int i = 0; i < 9; ++i) g[i] = buf[src_offset(i, x, y, a)];
+        double dr = g[0];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) f[i * n + k] = g[i] + shift_of(i, a.rho0, a.urx, a.ury);
+        for (int i = 1; i < 9; ++i) dr += g[i];
+        if (!finite(dr)) {
+            moments_plain(g, a, o, k);
+            continue;
         }
-        if (o.any()) {
-            if (isfinite(dr)) moments_plain<false>(g, a, o, k);
-            else moments_plain<true>(g, a, o, k);
-        }
+        double jx = 0, jy = 0, sxx = 0, sxy = 0, syy = 0;
+        if (o.ux) jx = g[1] - g[3] + g[5] - g[6] - g[7] + g[8];
+        if (o.uy) jy = g[2] - g[4] + g[5] + g[6] - g[7] - g[8];
+        if (o.pxx) sxx = g[1] + g[3] + g[5] + g[6] + g[7] + g[8];
+        if (o.pxy) sxy = g[5] - g[6] + g[7] - g[8];
+        if (o.pyy) syy = g[2] + g[4] + g[5] + g[6] + g[7] + g[8];
+        moments_close(dr, jx, jy, sxx, sxy, syy, a, o, k);
     }
 }
 
-// 32- and 16-bit storage: two neighbouring nodes per thread, gathered as in the step kernels.
 // shift: the constants s_i; second: ur_x^2 + c_s^2, rho0 ur_x, ur_y^2 + c_s^2.
 struct GatherConsts {
     double shift[9], second[3];
 };
+
+// Populations out, f = g + s: one node per thread, so that a warp stores 256 bytes in a row; bound by
+// these stores.
 template <typename S>
-__global__ void __launch_bounds__(kBlock) gather_kernel(const S* buf, FieldArgs a, double* f, MomentOut o, GatherConsts c) {
+__global__ void __launch_bounds__(kBlock) populations_kernel(const S* buf, FieldArgs a, double* f, GatherConsts c) {
     if (a.which && *a.which) buf += a.other;
-    const long long n = (long long)a.nx * a.ny;
+    const unsigned n = (unsigned)a.nx * (unsigned)a.ny;
+    if constexpr (sizeof(S) == 8)   // as scatter_kernel takes them off again, to the last place
+        if (a.urx != 0.0 || a.ury != 0.0) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) c.shift[i] = shift_of(i, a.rho0, a.urx, a.ury);
+        }
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int y = (int)(k / (unsigned)a.nx), x = (int)(k - (unsigned)y * (unsigned)a.nx);
+        S g[9];   // (loads first: a store to f might be one to buf, for all the compiler knows)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) g[i] = buf[src_offset(i, x, y, a)];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            if constexpr (sizeof(S) == 8) f[i * (long long)n + k] = g[i] + c.shift[i];
+            else f[i * (long long)n + k] = widen(Conv<S>::to_T(g[i])) + c.shift[i];
+        }
+    }
+}
+
+// Moments of 32- and 16-bit storage: two neighbouring nodes per thread, gathered as in the step kernels.
+template <typename S>
+__global__ void __launch_bounds__(kBlock) moments_kernel(const S* buf, FieldArgs a, MomentOut o, GatherConsts c) {
     const int lane = threadIdx.x & 31, nseg = (a.nx + 1) / 2;
     const bool shifted = a.urx != 0.0 || a.ury != 0.0;
     const unsigned total = (unsigned)a.ny * (unsigned)nseg, stride = gridDim.x * blockDim.x;
@@ -223,13 +246,6 @@ __global__ void __launch_bounds__(kBlock) gather_kernel(const S* buf, FieldArgs 
         gather_pull<S, 2, 1>(buf, a.nx, a.ny, a.pitch, a.plane, y, x0 / 2, nseg, x0, nvalid, lane, g);
         if (!active) continue;
         const long long k = (long long)y * a.nx + x0;
-        if (f) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i)
-                for (int j = 0; j < 2; ++j)
-                    if (j < nvalid) f[i * n + k + j] = widen(g[i][j]) + c.shift[i];
-        }
-        if (!o.any()) continue;
         F2 p[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) p[i] = f2_make(g[i][0], g[i][1]);
@@ -274,7 +290,7 @@ __global__ void __launch_bounds__(kBlock) gather_kernel(const S* buf, FieldArgs 
                 double d[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) d[i] = (double)g[i][j];
-                moments_plain<true>(d, a, o, k + j);
+                moments_plain(d, a, o, k + j);
                 continue;
             }
             if (o.rho) o.rho[k + j] = r;
@@ -622,17 +638,19 @@ cudaError_t scatter_t(void* buf, const FieldArgs& a, const double* f, cudaStream
 }
 template <typename S>
 cudaError_t gather_t(const void* buf, const FieldArgs& a, double* f, const MomentOut& o, cudaStream_t s) {
+    GatherConsts c;
+    for (int i = 0; i < 9; ++i) c.shift[i] = shift_of(i, a.rho0, a.urx, a.ury);
+    c.second[0] = std::fma(a.urx, a.urx, 1.0 / 3.0);
+    c.second[1] = a.rho0 * a.urx;
+    c.second[2] = std::fma(a.ury, a.ury, 1.0 / 3.0);
+    const Spread g = spread((long long)a.nx * a.ny);
+    if (f) populations_kernel<S><<<g.grid, g.block, 0, s>>>((const S*)buf, a, f, c);
+    if (!o.any()) return cudaGetLastError();
     if constexpr (sizeof(S) == 8) {
-        const Spread g = spread((long long)a.nx * a.ny);
-        gather_kernel_f64<<<g.grid, g.block, 0, s>>>((const double*)buf, a, f, o);
+        moments_kernel_f64<<<g.grid, g.block, 0, s>>>((const double*)buf, a, o);
     } else {
-        GatherConsts c;
-        for (int i = 0; i < 9; ++i) c.shift[i] = shift_of(i, a.rho0, a.urx, a.ury);
-        c.second[0] = std::fma(a.urx, a.urx, 1.0 / 3.0);
-        c.second[1] = a.rho0 * a.urx;
-        c.second[2] = std::fma(a.ury, a.ury, 1.0 / 3.0);
-        const Spread g = spread((long long)a.ny * ((a.nx + 1) / 2));
-        gather_kernel<S><<<g.grid, g.block, 0, s>>>((const S*)buf, a, f, o, c);
+        const Spread h = spread((long long)a.ny * ((a.nx + 1) / 2));
+        moments_kernel<S><<<h.grid, h.block, 0, s>>>((const S*)buf, a, o, c);
     }
     return cudaGetLastError();
 }
