@@ -90,6 +90,7 @@ struct lbm_group {
     struct Recorded {                  // a recorded graph, by the parity of the first context's buffer
         cudaGraphExec_t exec = nullptr;
         std::vector<int> parity;       // ctx->cur of each context when the graph was recorded
+        int flips = 0;                 // an odd number of launches: every context ends on the other buffer
         std::vector<unsigned> gen;     // ctx->gen of each context when the graph was recorded
     } rec[2];
     int timing = 0;
@@ -553,12 +554,8 @@ MarchPlan march_plan(const lbm_group* g, long long n) {
 // what the one-step kernels are for).
 bool use_march(const lbm_group* g, long long n) { return g->march > 1 && n >= 2 && tile_shift(g) >= 0; }
 
-// Time-fused launches of a run of n steps, t at most in each; `even` (a recorded graph, which must
-// end on the buffers it began with) one more if that is odd.
-long long march_launches(long long n, int t, bool even) {
-    const long long l = (n + t - 1) / t;
-    return even && l % 2 ? l + 1 : l;
-}
+// Time-fused launches of a run of n steps, t at most in each.
+long long march_launches(long long n, int t) { return (n + t - 1) / t; }
 
 // One time-fused launch: t time steps of every context by plan p.
 int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
@@ -597,11 +594,11 @@ int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
 
 // n time steps of the group: time-fused launches where the group has them, else bulk-copy
 // launches for a tiled group, else n launches
-int group_advance(lbm_group* g, cudaStream_t s, long long n, bool even = false) {
+int group_advance(lbm_group* g, cudaStream_t s, long long n) {
     if (n <= 0) return LBM_OK;
     if (use_march(g, n)) {
         const MarchPlan p = march_plan(g, n);
-        const long long l = march_launches(n, p.t, even);
+        const long long l = march_launches(n, p.t);
         for (long long k = 0; k < l; ++k) {   // lengths differ by at most one step
             int rc = launch_march(g, s, (int)(n / l + (k < n % l ? 1 : 0)), p);
             if (rc != LBM_OK) return rc;
@@ -700,16 +697,20 @@ int group_record(lbm_group* g) {
         cudaGraphExecDestroy(R.exec);
         R.exec = nullptr;
     }
-    // record on the private stream; the buffers alternate, so after an even number of launches
-    // every context is back on the buffer it started from and the graph can be replayed
+    // Record on the private stream.  The buffers alternate, so after an odd number of launches
+    // (time-fused ones; the others' parity is that of the even number of steps) every context is on
+    // the other buffer, where the graph of that parity goes on: a launch more to make it even would be
+    // one of fewer steps (a graph of 2 steps as two launches of one took 1.2-1.5x the time of the
+    // one-step kernels on three 4096^2 lattices).
     std::vector<int> cur0(g->ctx.size());
     std::vector<long long> steps0(g->ctx.size());
     for (size_t k = 0; k < g->ctx.size(); ++k) { cur0[k] = g->ctx[k]->cur; steps0[k] = g->ctx[k]->steps; }
     LBM_CK(c0, cudaStreamBeginCapture(g->capture, cudaStreamCaptureModeThreadLocal));
     int rc = LBM_OK;
-    rc = group_advance(g, g->capture, g->graph_steps, true);
+    rc = group_advance(g, g->capture, g->graph_steps);
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(g->capture, &graph);
+    R.flips = c0->cur != cur0[0] ? 1 : 0;
     for (size_t k = 0; k < g->ctx.size(); ++k) { g->ctx[k]->cur = cur0[k]; g->ctx[k]->steps = steps0[k]; }
     if (rc != LBM_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -757,12 +758,15 @@ int group_replay(lbm_group* g) {
         LBM_CK(c0, cudaEventRecord(e1, g->stream));
         g->pending_lattice_steps += (long long)g->graph_steps * (long long)g->ctx.size();
         g->pending_kernels += use_march(g, g->graph_steps)
-                                  ? march_launches(g->graph_steps, march_plan(g, g->graph_steps).t, true)
+                                  ? march_launches(g->graph_steps, march_plan(g, g->graph_steps).t)
                               : (g->tiled && tile_shift(g) >= 0)
                                   ? (long long)(g->graph_steps + tile_steps_per_launch(g) - 1) / tile_steps_per_launch(g)
                                   : (long long)g->graph_steps * (g->fused ? 1LL : (long long)g->ctx.size());
     }
-    for (lbm_ctx* c : g->ctx) c->steps += g->graph_steps;   // even: buffers end where they began
+    for (lbm_ctx* c : g->ctx) {
+        c->cur ^= R.flips;
+        c->steps += g->graph_steps;
+    }
     return LBM_OK;
 }
 
