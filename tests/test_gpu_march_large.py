@@ -1,6 +1,7 @@
 """Time-fused launches of large lattices: whole waves of tall marches, four steps each, in the unrolled
-form (one model) and the rolled one (several), over even and odd rows, against the register-staged
-kernels, bit for bit.  No tolerance is involved."""
+form (one model) and the rolled one (several), over even and odd rows -- against the register-staged
+kernels, bit for bit -- and the copy-engine launches that the library's own choice took before it
+marched.  No tolerance is involved."""
 
 import pytest
 
@@ -80,3 +81,47 @@ def test_tall_marches_of_four_steps(L, shape, models, storage, shift):
     L.lbm_group_destroy(g)
     for lat in fused + plain:
         lat.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("models", [MODELS, ["bgk", "rm", "hm", "pr"]])
+def test_copy_engine_group_of_1024_lattices(L, models, storage):
+    """The benchmark's group of 1024 x 1024 lattices in one copy-engine launch a step."""
+    staged = _lattices(L, (1024, 1024), models, storage, False, L.LBM_PATH_BULK)
+    plain = _lattices(L, (1024, 1024), models, storage, False, L.LBM_PATH_VECTOR)
+    g = L.lbm_group_create([x.ctx for x in staged], graph_steps=8)
+    assert L.lbm_group_describe(g)["family"] == L.LBM_PATH_BULK
+    L.lbm_group_step(g, 21)
+    for m, a, b in zip(models, staged, plain):
+        b.step(21)
+        assert _same(a, b), m
+        assert a.status() == (L.LBM_OK, -1, 21)
+    L.lbm_group_destroy(g)
+    for lat in staged + plain:
+        lat.close()
+
+
+@pytest.mark.parametrize("storage", ["f16", "bf16"])
+def test_copy_engine_at_16384(L, storage):
+    """The 16384 x 16384 16-bit lattice, one copy-engine launch a step: rho and u of every node."""
+    n = 16384
+    x = torch.arange(n, device="cuda", dtype=torch.float64) * (2 * np.pi / n)
+    ux = 0.1 + 0.05 * torch.sin(3 * x)[:, None] * torch.cos(5 * x)[None, :]
+    uy = 0.04 * torch.cos(2 * x)[:, None] * torch.sin(7 * x)[None, :]
+    rho = torch.ones_like(ux)
+    out = []
+    for path in (L.LBM_PATH_BULK, L.LBM_PATH_VECTOR):
+        lat = L.Lattice(n, n, "chm", RATES, storage=L.STORAGES[storage])
+        lat.set_shift_velocity(0.1, 0.0)
+        lat.set_kernel_path(path)
+        lat.init_equilibrium(rho, ux, uy)
+        lat.step(8)
+        assert lat.status()[0] == L.LBM_OK
+        fields = [torch.empty_like(ux) for _ in range(3)]
+        lat.moments(*fields)
+        lat.close()
+        out.append(fields)
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+    del out, fields, rho, ux, uy
+    torch.cuda.empty_cache()
