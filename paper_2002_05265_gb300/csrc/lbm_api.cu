@@ -280,9 +280,10 @@ int ensure_stage(lbm_ctx* c, size_t elems) {
     return LBM_OK;
 }
 
-// Launch with programmatic stream serialization: the kernel is scheduled while its predecessor on
-// the stream still runs, and waits for it by itself (griddepcontrol.wait) before it touches memory.
-cudaError_t launch_dependent(const void* kernel, int grid, int block, int smem, void** args, cudaStream_t s) {
+// Launch that may, with `overlap`, be scheduled while its predecessor on the stream still runs
+// (programmatic stream serialization): the kernel waits for it by itself (griddepcontrol.wait) before
+// it touches memory.
+cudaError_t launch_kernel(const void* kernel, int grid, int block, int smem, void** args, cudaStream_t s, bool overlap) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
@@ -290,18 +291,32 @@ cudaError_t launch_dependent(const void* kernel, int grid, int block, int smem, 
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 
-int launch_step_once(lbm_ctx* c, cudaStream_t s) {
+// Whether register-staged steps overlap their launches.  What it saves is the launch latency; what it
+// costs is the even spread of the CTAs over the SMs, since those of the next launch take the places
+// as they come free.  Two launches of a warp for every second scheduler fit side by side (128 x 37 FP64
+// BGK 3.46 against 3.59 us a step, recorded); more warps in recorded steps, whose latency is short, lose
+// by it (FP64 BGK 128^2 5.51 against 3.97 us, 256^2 of second order 38 against 20.6, FP16 1001 x 777 7.6
+// against 6.2), and FP64 steps, which wait for the busiest scheduler's pipe, lose launched one by one
+// too (160^2 14.5 against 7.5); FP32 and 16-bit steps launched one by one gain (512^2 4.7 against 6.2,
+// 1001 x 777 K 7.9 against 8.5).
+bool overlap_steps(int storage, int grid, int block, bool recorded) {
+    const long long warps = (long long)grid * block / 32;
+    return warps <= 2 * 152 || (!recorded && storage != LBM_F64);
+}
+
+int launch_step_once(lbm_ctx* c, cudaStream_t s, bool recorded) {
     StepArgs a = step_args(c);
     const void* src = c->buf[c->cur];
     void* dst = c->buf[c->cur ^ 1];
     void* args[] = {(void*)&src, (void*)&dst, (void*)&a};
-    LBM_CK(c, launch_dependent(c->kernel, c->grid, c->block, 0, args, s));
+    LBM_CK(c, launch_kernel(c->kernel, c->grid, c->block, 0, args, s,
+                            overlap_steps(c->storage, c->grid, c->block, recorded)));
     c->cur ^= 1;
     c->steps += 1;
     return LBM_OK;
@@ -309,7 +324,7 @@ int launch_step_once(lbm_ctx* c, cudaStream_t s) {
 
 // one time step of every context of a fused group, as one multi-lattice launch (all contexts
 // must agree on the default vs reference-velocity shift)
-int launch_group_once(lbm_group* g, cudaStream_t s, int sh) {
+int launch_group_once(lbm_group* g, cudaStream_t s, int sh, bool recorded) {
     lbm::GroupArgs ga;
     ga.n = (int)g->ctx.size();
     ga.padded_total = g->padded_total;
@@ -325,7 +340,8 @@ int launch_group_once(lbm_group* g, cudaStream_t s, int sh) {
         e.total = (unsigned)c->ny * (unsigned)c->nseg;
     }
     void* args[] = {(void*)&ga};
-    LBM_CK(g->ctx[0], launch_dependent(g->gkernel[sh], g->ggrid[sh], g->gblock, 0, args, s));
+    LBM_CK(g->ctx[0], launch_kernel(g->gkernel[sh], g->ggrid[sh], g->gblock, 0, args, s,
+                                    overlap_steps(g->ctx[0]->storage, g->ggrid[sh], g->gblock, recorded)));
     for (lbm_ctx* c : g->ctx) {
         c->cur ^= 1;
         c->steps += 1;
@@ -451,15 +467,16 @@ int tile_shift(const lbm_group* g) {
 }
 
 int group_step_once(lbm_group* g, cudaStream_t s) {
+    const bool recorded = g->capture && s == g->capture;
     if (g->tiled && tile_shift(g) >= 0) return launch_tile_steps(g, s, tile_shift(g), 1);
     if (g->fused) {
         int nsh = 0;
         for (lbm_ctx* c : g->ctx) nsh += is_shifted(c) ? 1 : 0;
-        if (nsh == 0) return launch_group_once(g, s, 0);
-        if (nsh == (int)g->ctx.size()) return launch_group_once(g, s, 1);
+        if (nsh == 0) return launch_group_once(g, s, 0, recorded);
+        if (nsh == (int)g->ctx.size()) return launch_group_once(g, s, 1, recorded);
     }
     for (lbm_ctx* c : g->ctx) {
-        int rc = launch_step_once(c, s);
+        int rc = launch_step_once(c, s, recorded);
         if (rc != LBM_OK) return rc;
     }
     return LBM_OK;
@@ -584,7 +601,7 @@ int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
         for (int j = 0; j < lbm::kNumConsts; ++j) e.c[j] = make_float2(a.cf[j], a.cf[j]);
     }
     void* args[] = {(void*)&ma};
-    LBM_CK(g->ctx[0], launch_dependent(g->mkernel[tile_shift(g)], (int)begin, 32 * p.per, g->msmem * p.per, args, s));
+    LBM_CK(g->ctx[0], launch_kernel(g->mkernel[tile_shift(g)], (int)begin, 32 * p.per, g->msmem * p.per, args, s, true));
     for (lbm_ctx* c : g->ctx) {
         c->cur ^= 1;
         c->steps += t;
