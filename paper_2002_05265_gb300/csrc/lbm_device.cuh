@@ -262,6 +262,10 @@ __device__ __forceinline__ F2 mul(F2 a, F2 b) {
 // instead lets the assembler fuse a product into the sum, which does not)
 __device__ __forceinline__ F2 sub(F2 a, F2 b) { return fma3(b, f2_make(-1.0f, -1.0f), a); }
 
+// -s for s = a + b, from -a and b: an operand sign for one node, an instruction for two
+__device__ __forceinline__ float negative(float s, float, float) { return -s; }
+__device__ __forceinline__ F2 negative(F2, F2 na, F2 b) { return sub(na, b); }
+
 // 1/x.  FP32: the hardware approximation (rcp.approx) refined by one Newton-Raphson step,
 // r' = r + r (1 - x r), two FMAs; within an ulp of the rounded quotient and free of any
 // data-dependent branch, so a lattice that has blown up (non-finite populations) steps as fast
@@ -307,9 +311,10 @@ __device__ __forceinline__ Consts<T> make_consts_table(const T* t) {
     Consts<T> c;
     c.w = t[0]; c.w3 = t[1]; c.w4 = t[2]; c.rho0 = t[3]; c.urx = t[4]; c.ury = t[5];
     c.Xr = t[12]; c.Yr = t[13];
-    c.ka = t[14]; c.kb = t[15]; c.nkb = t[26];
-    c.nrho0 = t[18];
-    c.nw = t[27]; c.nw3 = t[28]; c.nw4 = t[29];
+    c.ka = t[14]; c.kb = t[15];
+    // (the entries 18, 26-29, as operand signs)
+    c.nkb = -c.kb; c.nrho0 = -c.rho0;
+    c.nw = -c.w; c.nw3 = -c.w3; c.nw4 = -c.w4;
     c.ww3 = t[19]; c.rr = t[20]; c.qq = t[21];
     c.sw4 = t[22];
     c.nc3 = t[23]; c.nc4 = t[24]; c.sw1 = t[25];
@@ -526,7 +531,7 @@ __device__ __forceinline__ void collide_f32(const P (&g)[9], P (&o)[9], const Co
     P jx = add(add(a1p, a1z), a1m), jy = sub(a0p, a0m);
     const P m20 = add(add(a2p, a2z), a2m), m02 = add(a0p, a0m), m11 = sub(a1p, a1m);
     const P m21 = sub(a2p, a2m), m12 = add(a1p, a1m), m22 = add(a2p, a2m);
-    const P rho = add(drho, c.rho0), nrho = sub(c.nrho0, drho);
+    const P rho = add(drho, c.rho0), nrho = negative(rho, c.nrho0, drho);
     if (SHIFT) {
         jx = fma3(c.rho0, c.urx, jx);
         jy = fma3(c.rho0, c.ury, jy);
