@@ -299,15 +299,15 @@ cudaError_t launch_kernel(const void* kernel, int grid, int block, int smem, voi
 
 // Whether register-staged steps overlap their launches.  What it saves is the launch latency; what it
 // costs is the even spread of the CTAs over the SMs, since those of the next launch take the places
-// as they come free.  Two launches of a warp for every second scheduler fit side by side (128 x 37 FP64
-// BGK 3.46 against 3.59 us a step, recorded); more warps in recorded steps, whose latency is short, lose
+// as they come free.  Two launches of a warp for every second scheduler fit side by side (67 x 37 FP64
+// BGK 3.46 against 3.65 us a step, recorded; launched one by one a few more do, 100^2 4.6 against 6.2); more warps in recorded steps, whose latency is short, lose
 // by it (FP64 BGK 128^2 5.51 against 3.97 us, 256^2 of second order 38 against 20.6, FP16 1001 x 777 7.6
 // against 6.2), and FP64 steps, which wait for the busiest scheduler's pipe, lose launched one by one
 // too (160^2 14.5 against 7.5); FP32 and 16-bit steps launched one by one gain (512^2 4.7 against 6.2,
-// 1001 x 777 K 7.9 against 8.5).
-bool overlap_steps(int storage, int grid, int block, bool recorded) {
+// 1001 x 777 K 7.9 against 8.5), unless a warp takes several rows (3 x 30,000 FP32 17 against 8).
+bool overlap_steps(int storage, int grid, int block, int nseg, bool recorded) {
     const long long warps = (long long)grid * block / 32;
-    return warps <= 2 * 152 || (!recorded && storage != LBM_F64);
+    return warps <= (recorded ? 304 : 400) || (!recorded && storage != LBM_F64 && nseg >= 32);
 }
 
 int launch_step_once(lbm_ctx* c, cudaStream_t s, bool recorded) {
@@ -316,7 +316,7 @@ int launch_step_once(lbm_ctx* c, cudaStream_t s, bool recorded) {
     void* dst = c->buf[c->cur ^ 1];
     void* args[] = {(void*)&src, (void*)&dst, (void*)&a};
     LBM_CK(c, launch_kernel(c->kernel, c->grid, c->block, 0, args, s,
-                            overlap_steps(c->storage, c->grid, c->block, recorded)));
+                            overlap_steps(c->storage, c->grid, c->block, c->nseg, recorded)));
     c->cur ^= 1;
     c->steps += 1;
     return LBM_OK;
@@ -340,8 +340,11 @@ int launch_group_once(lbm_group* g, cudaStream_t s, int sh, bool recorded) {
         e.total = (unsigned)c->ny * (unsigned)c->nseg;
     }
     void* args[] = {(void*)&ga};
+    // (recorded launches of several lattices gain nothing at any size: four 33 x 31 FP16 4.5 against 3.5 us)
+    int nseg = g->ctx[0]->nseg;
+    for (const lbm_ctx* c : g->ctx) nseg = std::min(nseg, c->nseg);
     LBM_CK(g->ctx[0], launch_kernel(g->gkernel[sh], g->ggrid[sh], g->gblock, 0, args, s,
-                                    overlap_steps(g->ctx[0]->storage, g->ggrid[sh], g->gblock, recorded)));
+                                    !recorded && overlap_steps(g->ctx[0]->storage, g->ggrid[sh], g->gblock, nseg, recorded)));
     for (lbm_ctx* c : g->ctx) {
         c->cur ^= 1;
         c->steps += 1;
@@ -1254,9 +1257,14 @@ int lbm_group_create(lbm_group** out, lbm_ctx* const* ctxs, int n, int graph_ste
             off += (segs + 31u) / 32u * 32u;
         }
         g->padded_total = off;
+        bool models = false;
+        for (int k = 1; k < n; ++k) models = models || kernel_model(ctxs[k]->model) != kernel_model(ctxs[0]->model);
         for (int sh = 0; sh < 2; ++sh) {
             g->gkernel[sh] = pick_group_kernel(ctxs[0]->storage, sh == 1);
-            g->gblock = lbm::spread_block(off);
+            // (16-bit lattices of several models: whole CTAs, so that an SM's warps share a model's code;
+            // four 257 x 255 of different models 4.3 us a step, in CTAs of 64 threads 7.2)
+            const bool whole = models && lbm::storage_bytes(ctxs[0]->storage) == 2 && off >= 16384;
+            g->gblock = whole ? 256 : lbm::spread_block(off);
             g->ggrid[sh] = resident_grid(g->gkernel[sh], g->gblock, off);
         }
         g->fused = 1;
