@@ -81,6 +81,7 @@ struct lbm_group {
     int mgrid = 0;                     // their resident CTAs (of kMarchWarps warps)
     int msmem = 0;                     // their shared memory per warp
     int mixed = 0;                     // contexts of several models
+    int sms = 152;
     cudaStream_t stream = nullptr;
     cudaStream_t capture = nullptr;
     std::vector<cudaStream_t> side;    // concurrent blow-up checks (launch_checks)
@@ -533,6 +534,26 @@ struct MarchPlan {
     int per;   // warps of a CTA
 };
 
+// Weight of the group's lattices when t steps are fused: strip rows by cost.
+double march_work(const lbm_group* g, int t) {
+    const int width = lbm::march_width(t);
+    double work = 0.0;
+    for (const lbm_ctx* c : g->ctx) work += (double)((c->nx + width - 1) / width) * c->ny * march_cost(c->model);
+    return work;
+}
+// Bands of a lattice: by its share of the work, so that every march costs about the same.
+int march_bands(const lbm_ctx* c, const MarchPlan& p, double work) {
+    const double bands = (double)p.warps * c->ny * march_cost(c->model) / work;
+    return std::max(1, std::min(c->ny, (int)bands));
+}
+long long march_ctas(const lbm_group* g, const MarchPlan& p, double work) {
+    const int width = lbm::march_width(p.t);
+    long long ctas = 0;
+    for (const lbm_ctx* c : g->ctx)
+        ctas += ((long long)((c->nx + width - 1) / width) * march_bands(c, p, work) + p.per - 1) / p.per;
+    return ctas;
+}
+
 // Large lattices fuse as many steps as the kernel has levels, in whole waves of resident warps
 // that march 80-160 rows: shorter, and the t - 1 rows each level recomputes weigh; longer, and
 // neighbouring marches drift apart and lose each other's lines (16384^2 FP32 K against 128 rows:
@@ -545,9 +566,14 @@ struct MarchPlan {
 // on 304 2.5, on 2432 3.3; 512^2: t = 2 on 1216 2.9, t = 4 on 2432 4.0; 128^2: t = 3 on 384 1.5).
 MarchPlan march_plan(const lbm_group* g, long long n) {
     const long long slots = (long long)g->mgrid * lbm::kMarchWarps, scheds = slots / 4;
-    const int most = (int)std::min<long long>(g->march, n);
-    const long long rows = march_strip_rows(g, most);
+    int most = (int)std::min<long long>(g->march, n);
+    long long rows = march_strip_rows(g, most);
     if (most == g->march && rows >= 24 * slots) {
+        // two steps a launch, whose strips are 60 columns wide, where that saves a strip worth more than
+        // the second half of the fusion (57-60 columns: 500,000 rows in BF16 296 -> 218 us, 100,000 in
+        // FP32 56 -> 52; 2048^2: FP32 27.5 against 21.4, FP16 23.8 against 22.2)
+        const double dearer = g->ctx[0]->storage == LBM_F32 ? 1.55 : 1.13;
+        if (dearer * (double)march_strip_rows(g, 2) < (double)rows) rows = march_strip_rows(g, most = 2);
         long long waves = (rows + 160 * slots - 1) / (160 * slots);
         if (g->mixed && waves < 2 && rows >= 48 * slots) waves = 2;
         return {most, slots * waves, lbm::kMarchWarps};
@@ -570,9 +596,67 @@ MarchPlan march_plan(const lbm_group* g, long long n) {
     return best;
 }
 
-// Whether a run of n steps takes the time-fused launches (at least two steps: a single one is
-// what the one-step kernels are for).
-bool use_march(const lbm_group* g, long long n) { return g->march > 1 && n >= 2 && tile_shift(g) >= 0; }
+// Estimated time of a step in the time-fused launches of plan p, us: the model of march_plan with the
+// CTAs as they fall on the SMs.  Single 4-byte copies (odd rows; 16-bit ones not even asynchronous),
+// the shift and the models' operations as measured (14 and 15 columns, 300,000 rows, K: FP32 75.4 and
+// 85.7 us a step, FP16 78.5 and 98.3; 4096^2 K FP32 77 us, with shift 91).
+double march_us(const lbm_group* g, const MarchPlan& p) {
+    const double work = march_work(g, p.t);
+    const long long ctas = march_ctas(g, p, work);
+    int rows = 1, odd = 0;
+    double nodes = 0.0, cost = 0.0;
+    for (const lbm_ctx* c : g->ctx) {
+        const int bands = march_bands(c, p, work);
+        rows = std::max(rows, (c->ny + bands - 1) / bands);
+        odd |= c->nx & 1;
+        nodes += (double)c->nx * c->ny;
+        cost += (double)c->nx * c->ny * march_cost(c->model);
+    }
+    const int room = 2 * lbm::kMarchWarps / p.per;   // CTAs an SM holds
+    const double load = std::min<double>(room, (double)((ctas + g->sms - 1) / g->sms)) * p.per / 4;   // warps a scheduler
+    const double waves = std::max(1.0, (double)ctas / ((double)g->sms * room));
+    const double each = load <= 1 ? 0.25 : (load <= 2 ? 0.14 + 0.11 * load : 0.36 + (load - 2) * (0.06 + 0.24 / p.t));
+    const int storage = g->ctx[0]->storage;
+    double f = odd ? (storage == LBM_F32 ? 1.12 : (storage == LBM_F16 ? 1.33 : 1.25)) : 1.02;
+    f *= 0.5 + 0.5 * cost / (nodes * march_cost(LBM_K));
+    if (tile_shift(g) == 1) f *= 1.1;
+    return f * (2.2 + each * p.t * (rows + p.t - 1) * waves) / p.t;
+}
+
+// Estimated time of a step in the register-staged kernels, us, from 460 lattices of 3 to 4095 columns
+// and 3 to 300,000 rows: threads, a warp's rows (each a line of its own), an odd number of vectors a
+// row, and beyond the L2 the sectors a row touches.  Launched one by one a step waits longer.
+double staged_us(const lbm_group* g, bool recorded) {
+    const bool f32 = g->ctx[0]->storage == LBM_F32;
+    const int s = f32 ? 4 : 2, granule = f32 ? 64 : 32;
+    double threads = 0.0, latency = 0.0, lines = 0.0, bytes = 0.0;
+    bool uneven = false;   // an odd number of vectors a row: warps start anywhere in a row
+    for (const lbm_ctx* c : g->ctx) {
+        const bool odd = c->nseg % 2 && c->nseg > 1 && c->nseg < 32;
+        uneven |= odd;
+        threads += (double)c->ny * c->nseg * (odd ? (f32 ? 1.4 : 1.15) : 1.0);
+        latency = std::max(latency, (f32 ? 3.5 : 1.8) / c->nseg);
+        const long long row = (long long)c->nx * s;
+        lines += 18.0 * c->ny * (double)((row + 127) / 128 * 128);
+        const double sectors = 18.0 * c->ny * (double)((row + granule - 1) / granule * granule);
+        bytes += sectors * (row <= 512 ? (f32 ? 1.54 : 1.04) : 1.0) * (odd ? (f32 ? 1.8 : 1.25) : 1.0);
+    }
+    double us = latency + (f32 ? 1.7 + 26.5e-6 * threads : std::max(2.4 + 36e-6 * threads, 1.0 + 53.5e-6 * threads));
+    if (lines > (uneven ? 130e6 : 140e6)) us = std::max(us, bytes / (f32 ? 6.0e6 : 5.0e6));
+    return recorded ? us : us + 1.5;
+}
+
+// Whether a run of n steps takes the time-fused launches: at least two steps (a single one is what
+// the one-step kernels are for), and where the register-staged kernels are what it would take
+// otherwise, not if those are quicker: lattices of few columns or few rows, of which a march keeps
+// little, and odd 16-bit ones that stay in the L2 (us a step, register-staged against fused: FP16
+// 3 x 100,000 16 / 36, 57 x 3000 2.9 / 3.5, 701 x 699 4.6 / 5.8, 1,000,001 x 4 30 / 40; FP32
+// 21 x 30,000 6.8 / 11.2).  The copy-engine kernels, which rows of whole 16-byte chunks take
+// otherwise, are slower everywhere.
+bool use_march(const lbm_group* g, long long n, bool recorded) {
+    if (!(g->march > 1 && n >= 2 && tile_shift(g) >= 0)) return false;
+    return g->tiled || 0.95 * march_us(g, march_plan(g, n)) < staged_us(g, recorded);
+}
 
 // Time-fused launches of a run of n steps, t at most in each.
 long long march_launches(long long n, int t) { return (n + t - 1) / t; }
@@ -583,9 +667,9 @@ int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
     ma.n = (int)g->ctx.size();
     ma.t = t;
     const int width = lbm::march_width(t);
-    double work = 0.0;
-    for (const lbm_ctx* c : g->ctx) work += (double)((c->nx + width - 1) / width) * c->ny * march_cost(c->model);
+    const double work = march_work(g, t);
     unsigned begin = 0;
+    int rows = 1;
     for (size_t k = 0; k < g->ctx.size(); ++k) {
         lbm_ctx* c = g->ctx[k];
         lbm::MarchEntry& e = ma.e[k];
@@ -595,16 +679,19 @@ int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
         e.nx = c->nx; e.ny = c->ny; e.pitch = c->pitch;
         e.model = kernel_model(c->model);
         e.strips = (c->nx + width - 1) / width;
-        // bands by the lattice's share of the work, so that every march costs about the same
-        const double bands = (double)p.warps * c->ny * march_cost(c->model) / work;
-        e.bands = std::max(1, std::min(c->ny, (int)bands));
+        e.bands = march_bands(c, p, work);
+        rows = std::max(rows, (c->ny + e.bands - 1) / e.bands);
         e.begin = begin;
         begin += (unsigned)((e.strips * (long long)e.bands + p.per - 1) / p.per);
         const StepArgs a = step_args(c);
         for (int j = 0; j < lbm::kNumConsts; ++j) e.c[j] = make_float2(a.cf[j], a.cf[j]);
     }
     void* args[] = {(void*)&ma};
-    LBM_CK(g->ctx[0], launch_kernel(g->mkernel[tile_shift(g)], (int)begin, 32 * p.per, g->msmem * p.per, args, s, true));
+    // Launches overlap (overlap_steps), but not those that leave SMs idle and march several rows: the next
+    // launch's CTAs would share the idle SMs (30,000 x 10, 134 CTAs, recorded: 4.8 against 3.5 us a step)
+    const bool recorded = g->capture && s == g->capture;
+    const bool overlap = begin >= (unsigned)g->sms || rows <= (recorded ? 2 : 6);
+    LBM_CK(g->ctx[0], launch_kernel(g->mkernel[tile_shift(g)], (int)begin, 32 * p.per, g->msmem * p.per, args, s, overlap));
     for (lbm_ctx* c : g->ctx) {
         c->cur ^= 1;
         c->steps += t;
@@ -616,7 +703,7 @@ int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
 // launches for a tiled group, else n launches
 int group_advance(lbm_group* g, cudaStream_t s, long long n) {
     if (n <= 0) return LBM_OK;
-    if (use_march(g, n)) {
+    if (use_march(g, n, g->capture && s == g->capture)) {
         const MarchPlan p = march_plan(g, n);
         const long long l = march_launches(n, p.t);
         for (long long k = 0; k < l; ++k) {   // lengths differ by at most one step
@@ -777,7 +864,7 @@ int group_replay(lbm_group* g) {
     if (g->timing) {
         LBM_CK(c0, cudaEventRecord(e1, g->stream));
         g->pending_lattice_steps += (long long)g->graph_steps * (long long)g->ctx.size();
-        g->pending_kernels += use_march(g, g->graph_steps)
+        g->pending_kernels += use_march(g, g->graph_steps, true)
                                   ? march_launches(g->graph_steps, march_plan(g, g->graph_steps).t)
                               : (g->tiled && tile_shift(g) >= 0)
                                   ? (long long)(g->graph_steps + tile_steps_per_launch(g) - 1) / tile_steps_per_launch(g)
@@ -1303,6 +1390,7 @@ int lbm_group_create(lbm_group** out, lbm_ctx* const* ctxs, int n, int graph_ste
             g->mgrid = sh == 0 ? sms * per_sm : std::min(g->mgrid, sms * per_sm);
         }
         if (march) g->march = march_most(ctxs[0]->storage);
+        g->sms = sms;
         g->mixed = mixed ? 1 : 0;
     }
     if (graph_steps > 0) {

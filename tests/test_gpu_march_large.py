@@ -125,3 +125,31 @@ def test_copy_engine_at_16384(L, storage):
         assert torch.equal(a, b)
     del out, fields, rho, ux, uy
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("shape,storage,launches", [
+    ((3, 30000), "f16", 4), ((3, 30000), "f32", 4), ((21, 30000), "f32", 4), ((15, 30000), "f16", 4),
+    ((1000001, 4), "f16", 4), ((701, 699), "f16", 4),
+    ((8, 100000), "f16", 1), ((24, 30000), "f32", 1), ((52, 30000), "f32", 1), ((2001, 1999), "f16", 1)])
+def test_narrow_and_flat_lattices_are_not_fused(L, shape, storage, launches):
+    """Launches of a recorded run of four steps, by shape, and the state they leave."""
+    nx, ny = shape
+    x, y = (torch.arange(n, device="cuda", dtype=torch.float64) * (2 * np.pi / n) for n in (nx, ny))
+    f = [1 + 0 * y[:, None] + 0 * x[None, :], 0.05 * torch.sin(y)[:, None] * torch.cos(x)[None, :],
+         0.04 * torch.cos(2 * y)[:, None] + 0 * x[None, :]]
+    lats = []
+    for path in (L.LBM_PATH_AUTO, L.LBM_PATH_VECTOR):
+        lat = L.Lattice(nx, ny, "k", RATES, storage=L.STORAGES[storage])
+        lat.set_kernel_path(path)
+        lat.init_equilibrium(*[v.contiguous() for v in f])
+        lats.append(lat)
+    g = L.lbm_group_create([lats[0].ctx], graph_steps=4)
+    L.lbm_group_set_timing(g)
+    L.lbm_group_step(g, 12)
+    lats[1].step(12)
+    assert _same(*lats)
+    _, steps, n = L.lbm_group_timing(g)
+    assert (steps, n) == (12, 3 * launches)
+    L.lbm_group_destroy(g)
+    for lat in lats:
+        lat.close()
