@@ -3,8 +3,9 @@
 // persistent launch (the numerical-stability study of Sec. 5b run as a batch).
 //
 // Stepping: FP32 and 16-bit instances take the time-fused marches of lbm_march.cuh between checks
-// (four steps per read and write of the instance, the collision in two-wide FP32 instructions);
-// the step that checks, and FP64, sweep the instance's vector segments once per step.
+// (four steps per read and write of the instance, the collision in two-wide FP32 instructions) where
+// that is quicker; the step that checks, instances too small, narrow or flat for a march or checked too
+// often, and FP64 sweep the instance's vector segments once per step.
 //
 // Scheduling: the grid holds as many CTAs as the GPU keeps resident.  Each CTA repeatedly
 // claims the next instance from a global counter (instances ordered largest first), and
@@ -27,10 +28,16 @@ struct BatchInstance {   // read-only during a run
     long long off;       // element offset of buffer 0 in the slab; buffer 1 at off + 9 * plane
     StepArgs a;          // geometry (nseg is recomputed for the kernel's VEC), rates, shift
     int model;           // lbm::Model
-    int pad;
+    int march_from;      // least check interval from which its steps are fused (batch_fused)
     double ke_ref, ke_factor;   // optional <|u|^2> > ke_factor * ke_ref criterion (ke_ref > 0)
     EquilibriumConsts eq;       // factors of the shift, for the initial state
 };
+
+constexpr int kNeverMarch = 0x7fffffff;
+// Whether the steps between checks are fused: where that is quicker (lbm_batch_api.cu, march_from).
+__host__ __device__ constexpr bool batch_fused(int march_from, int check_every) {
+    return (check_every > 0 ? check_every : kNeverMarch - 1) >= march_from;
+}
 
 struct BatchState {      // updated by the kernel, one per instance
     long long steps;     // time steps taken
@@ -46,7 +53,7 @@ constexpr double kPertFloor = 1e-20;   // <|u - u_ref|^2> below this counts as "
 // Time steps `t` .. `t + n` of one instance without a check, fused as in lbm_march.cuh: the CTA's
 // warps share its strips and bands of rows, and a block of up to four steps ends at a barrier.
 // Measured on 1024 instances of 32..256 squared for 1000 steps (FP32): 245 -> 147 ms (87 -> 147
-// GLUPS) with 16 warps a CTA, 162 ms with 8 (200 instances: 58 and 105 ms, hence the default); the
+// GLUPS) with 16 warps a CTA, 162 ms with 8 (200 instances: 58 and 105 ms); the
 // unrolled form, whose code outgrows the instruction cache here, 225 ms.  What bounds it: 84 % of the
 // columns and 84 % of the rows that are marched are kept, the rest of the time is the FP32 pipe's.
 template <int MODEL, typename S, int BLOCK, bool PAIRS>
@@ -84,7 +91,7 @@ __device__ __forceinline__ int batch_march(S* buf0, S* buf1, int cur, int n, con
     return cur;
 }
 
-template <int MODEL, typename S, int VEC, int BLOCK>
+template <int MODEL, typename S, int VEC, int BLOCK, bool FUSED>
 __device__ __forceinline__ void batch_instance_loop(S* buf0, S* buf1, const StepArgs& a,
                                                     const BatchInstance& I, BatchState& st, long long target,
                                                     int check_every, double growth, double (*s_red)[4],
@@ -97,6 +104,7 @@ __device__ __forceinline__ void batch_instance_loop(S* buf0, S* buf1, const Step
     long long t = st.steps;
     int cur = st.cur;
     const double nodes = (double)a.nx * (double)a.ny;
+    const bool fused = FUSED && batch_fused(I.march_from, check_every);
     while (t < target) {
         const bool check = (check_every > 0) && (t % check_every == 0);
         const S* src = cur ? buf1 : buf0;
@@ -136,10 +144,10 @@ __device__ __forceinline__ void batch_instance_loop(S* buf0, S* buf1, const Step
                 }
                 *s_stop = blown ? 1 : 0;
             }
-        } else if constexpr (sizeof(S) == 8) {
+        } else if (!fused) {
             for (unsigned base = threadIdx.x & ~31u; base < total; base += BLOCK)
                 step_segment<MODEL, 4, S, VEC, false, true>(src, dst, a, c, base + lane, total, lane, dg);
-        } else {
+        } else if constexpr (FUSED) {
             // up to the next check
             const long long next = check_every > 0 ? (t / check_every + 1) * (long long)check_every : target;
             const int n = (int)min(min(next, target) - t, (long long)(1 << 20));
@@ -159,10 +167,13 @@ __device__ __forceinline__ void batch_instance_loop(S* buf0, S* buf1, const Step
     }
 }
 
-template <typename S, int VEC, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, sizeof(S) == 8 ? 1 : 512 / BLOCK) batch_kernel(S* slab, const BatchInstance* __restrict__ inst,
-                                                      BatchState* state, const int* __restrict__ order, int n,
-                                                      int* queue, long long target, int check_every, double growth) {
+// FUSED: some instances march.  Without that code the kernel is half as long, which a launch of many
+// small instances of several models, whose warps run different code side by side, is quicker by (300
+// of 32^2 FP32 2.8 us a step, with it 4.0).
+template <typename S, int VEC, int BLOCK, bool FUSED>
+__global__ void __launch_bounds__(BLOCK, FUSED ? 512 / BLOCK : 1)
+    batch_kernel(S* slab, const BatchInstance* __restrict__ inst, BatchState* state, const int* __restrict__ order, int n,
+                 int* queue, long long target, int check_every, double growth) {
     __shared__ int s_id;
     __shared__ int s_stop;
     __shared__ double s_red[BLOCK / 32][4];
@@ -184,14 +195,14 @@ __global__ void __launch_bounds__(BLOCK, sizeof(S) == 8 ? 1 : 512 / BLOCK) batch
             S* b0 = slab + I.off;
             S* b1 = b0 + 9 * a.plane;
             switch (I.model) {
-                case BGK: batch_instance_loop<BGK, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
-                case RM: batch_instance_loop<RM, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
-                case HM: batch_instance_loop<HM, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
-                case CM: batch_instance_loop<CM, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
-                case CHM: batch_instance_loop<CHM, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
-                case CUM: batch_instance_loop<CUM, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
-                case PR: batch_instance_loop<PR, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
-                default: batch_instance_loop<RR, S, VEC, BLOCK>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                case BGK: batch_instance_loop<BGK, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                case RM: batch_instance_loop<RM, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                case HM: batch_instance_loop<HM, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                case CM: batch_instance_loop<CM, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                case CHM: batch_instance_loop<CHM, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                case CUM: batch_instance_loop<CUM, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                case PR: batch_instance_loop<PR, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
+                default: batch_instance_loop<RR, S, VEC, BLOCK, FUSED>(b0, b1, a, I, st, target, check_every, growth, s_red, &s_stop); break;
             }
         }
         __syncthreads();   // state written and s_id consumed before the next claim

@@ -7,8 +7,10 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <functional>
 #include <new>
 #include <numeric>
+#include <queue>
 #include <vector>
 
 #include "lbm.h"
@@ -36,6 +38,13 @@ struct lbm_batch {
     double* stage = nullptr;           // host-pointer staging for init (lazy)
     size_t stage_elems = 0;
     int vec = 0, block = 0, grid = 0;
+    bool fused = false;                // the kernel with the marches
+    int smem = 0;                      // its dynamic shared memory
+    int per_sm = 0, sms = 0;           // resident CTAs per SM of the kernel; SMs
+    bool models = false;               // instances of several models
+    bool own_shape = true;             // the shape is the library's choice
+    int shape_check = -1;              // check interval the kernel was chosen for
+    std::vector<int> order;            // largest instances first
     const void* kernel = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long g_target = -1;
@@ -65,12 +74,12 @@ int berr(lbm_batch* b, int code, const char* fmt, ...) {
                         "%s failed: %s", #call, cudaGetErrorString(e_));                         \
     } while (0)
 
-const void* pick_batch_kernel(int storage, int vec, int block) {
+const void* pick_batch_kernel(int storage, int vec, int block, bool fused) {
     switch (storage) {
         case LBM_F64: return lbm::batch_kernel_f64(vec, block);
-        case LBM_F32: return lbm::batch_kernel_f32(vec, block);
-        case LBM_F16: return lbm::batch_kernel_f16(vec, block);
-        case LBM_BF16: return lbm::batch_kernel_bf16(vec, block);
+        case LBM_F32: return lbm::batch_kernel_f32(vec, block, fused);
+        case LBM_F16: return lbm::batch_kernel_f16(vec, block, fused);
+        case LBM_BF16: return lbm::batch_kernel_bf16(vec, block, fused);
         default: return nullptr;
     }
 }
@@ -81,9 +90,65 @@ int batch_smem(int storage, int block) {
     return block / 32 * (storage == LBM_F32 ? lbm::march_smem_bytes<float, true> : lbm::march_smem_bytes<__half, true>);
 }
 
-void default_shape(int storage, int* vec, int* block) {
-    *vec = 16 / lbm::storage_bytes(storage);
-    *block = storage == LBM_F64 ? 256 : 512;
+// ---- which instances march, and how many threads a CTA has --------------------------------------
+// Estimated us a step of an instance with `block` threads, `resident` such CTAs at work on its SM;
+// `spill`: the instances at work together exceed the L2.  Fitted to 17 shapes of 16 x 16 to 256 x 256,
+// 3 x 2000 to 2000 x 3, alone and 152, 304, 608 at a time, FP32 and FP16, mostly within a tenth.
+// One step at a time: latency a sweep, then nodes at the rate of so many warps, of a full SM or of HBM.
+double one_step_us(const BatchInstance& I, int vec, int block, int resident, bool spill) {
+    const double nodes = (double)I.a.ny * ((I.a.nx + vec - 1) / vec * vec);
+    const double alone = 0.7 + nodes / (block >= 512 ? 1020.0 : (block >= 256 ? 850.0 : 630.0));
+    return std::max(alone, 0.8 + nodes * resident / (spill ? 630.0 : 1040.0));
+}
+// t steps fused, a step: rounds of the CTA's warps over strips and bands, as batch_march takes them.
+double fused_us(const BatchInstance& I, int block, int resident, int t) {
+    const int warps = block / 32, most = lbm::MarchForm<float>::TMAX;
+    const int strips = (I.a.nx + lbm::march_width(most) - 1) / lbm::march_width(most);
+    long long least = 1ll << 40;
+    int bands = 1;
+    for (int b = 1; b <= 2 * warps; ++b) {
+        const long long cost = ((long long)strips * b + warps - 1) / warps * ((I.a.ny + b - 1) / b + most - 1);
+        if (cost < least) {
+            least = cost;
+            bands = b;
+        }
+    }
+    const long long tasks = (long long)((I.a.nx + lbm::march_width(t) - 1) / lbm::march_width(t)) * bands;
+    const double rows = (double)((tasks + warps - 1) / warps) * ((I.a.ny + bands - 1) / bands + t - 1);
+    const int load = warps * resident;   // warps of the SM: a level row takes so long
+    const double row = load <= 4 ? 0.26 : (load <= 8 ? 0.36 : 0.69);
+    return 0.5 + rows * row * (0.8 + 0.8 / t);
+}
+// what a check adds to a step: the folds of the diagnostics in FP64
+double check_us(const BatchInstance& I, int block, int resident) {
+    const double nodes = (double)I.a.nx * I.a.ny;
+    if (block >= 512) return 7.1 + nodes / 1100.0;
+    return block >= 256 ? (resident > 1 ? 4.0 + nodes / 900.0 : 4.5 + nodes / 870.0) : 3.5 + nodes * resident / 1100.0;
+}
+int resident_ctas(const lbm_batch* b) { return std::max(1, std::min(b->per_sm, (b->n + b->sms - 1) / b->sms)); }
+bool spills(const lbm_batch* b) {
+    const double together = std::min<double>(b->n, (double)b->sms * resident_ctas(b)) / b->n;
+    return (double)b->slab_bytes * together > 110e6;
+}
+// one_step_us in the kernel of the batch's shape: accesses below 16 bytes, and instances of several
+// models on an SM or beside the marches, which cost one another the instruction cache (800 of 96^2 in
+// BF16: 256 threads 98 us against 61 fused, 128 threads 149 against 56).
+double sweep_us(const lbm_batch* b, const BatchInstance& I) {
+    const int resident = resident_ctas(b);
+    double us = one_step_us(I, b->vec, b->block, resident, spills(b));
+    if (b->vec * lbm::storage_bytes(b->storage) < 16) us *= 1.25;
+    if (!b->models) return us;
+    if (b->storage == LBM_F32) return us * (b->fused ? (resident > 1 ? 1.35 : 1.1) : 1.0);
+    return us * (resident > 1 ? 1.7 : (b->fused ? 1.25 : 1.0));
+}
+// Least check interval from which marching instance I is quicker (kNeverMarch: never): the fewest
+// steps t that pay fused are what lies between two checks.
+int march_from(const lbm_batch* b, const BatchInstance& I) {
+    int from = lbm::kNeverMarch;
+    if (!b->fused) return from;
+    const double one = sweep_us(b, I);
+    for (int t = lbm::MarchForm<float>::TMAX; t >= 1 && fused_us(I, b->block, resident_ctas(b), t) < one; --t) from = t + 1;
+    return from;
 }
 
 bool is_device_ptr(const void* p) {
@@ -95,24 +160,97 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-int set_shape(lbm_batch* b, int vec, int block) {
-    const void* k = pick_batch_kernel(b->storage, vec, block);
+// The kernel of (vec, block), with the marches or without, and what of it suits the instances.
+int set_shape(lbm_batch* b, int vec, int block, bool fused) {
+    const void* k = pick_batch_kernel(b->storage, vec, block, fused);
     if (!k) return berr(b, LBM_ERR_UNSUPPORTED, "no batch kernel with vec=%d block=%d for this storage", vec, block);
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, per_sm = 0;
     LBM_BCK(b, cudaGetDevice(&dev));
-    LBM_BCK(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int smem = batch_smem(b->storage, block);
+    LBM_BCK(b, cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev));
+    const int smem = fused ? batch_smem(b->storage, block) : 0;
     LBM_BCK(b, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     LBM_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     if (per_sm < 1) return berr(b, LBM_ERR_UNSUPPORTED, "batch kernel cannot be resident");
     b->kernel = k;
     b->vec = vec;
     b->block = block;
+    b->fused = fused;
+    b->smem = smem;
+    b->per_sm = per_sm;
     // resident CTAs only (a persistent grid); never more CTAs than instances
-    b->grid = std::min(sms * per_sm, b->n);
+    b->grid = std::min(b->sms * per_sm, b->n);
+    for (BatchInstance& I : b->inst) I.march_from = march_from(b, I);
     return LBM_OK;
 }
 
+// Estimated us a step of all instances in runs checked every `check_every` steps: each to the CTA that
+// is free first, largest first, as the queue hands them out.
+double shape_us(const lbm_batch* b, int check_every) {
+    const int resident = resident_ctas(b);
+    const int apart = check_every > 0 ? check_every : 1 << 20;   // steps from check to check
+    const int t = std::min(apart - 1, (int)lbm::MarchForm<float>::TMAX);
+    std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
+    double last = 0.0;
+    for (int i : b->order) {
+        const BatchInstance& I = b->inst[i];
+        const double one = sweep_us(b, I);
+        const double rest = lbm::batch_fused(I.march_from, check_every) ? fused_us(I, b->block, resident, t) : one;
+        double us = rest + (one - rest + check_us(I, b->block, resident)) / apart;
+        if ((int)busy.size() == b->grid) {
+            us += busy.top();
+            busy.pop();
+        }
+        busy.push(us);
+        last = std::max(last, us);
+    }
+    return last;
+}
+
+// The kernel for runs checked every `check_every` steps.  With the shape left to the library, CTAs of
+// 512 threads (FP64 256), or of 256 where that is clearly quicker: two of 256 overlap one another's
+// barriers, loads and checks, one of 512 has an instance done sooner (us a step, 512 / 256: 300 of
+// 32^2 3.7 / 2.8, 800 of 96^2 60 / 54, 200 of 32..128 squared 21 / 37, 1024 of 32..256 147 / 162).
+int choose_shape(lbm_batch* b, int check_every) {
+    if (b->kernel && (b->storage == LBM_F64 || b->shape_check == check_every)) return LBM_OK;
+    const int own = 16 / lbm::storage_bytes(b->storage), given = b->block, vec = b->own_shape ? own : b->vec;
+    struct {
+        int block;
+        bool fused;
+        double worth;
+    } best = {0, false, 1e300}, all[] = {{512, true, 1.0}, {512, false, 1.0}, {256, false, 1.0}, {256, true, 1.0}};
+    if (b->storage == LBM_F64) {
+        best.block = 256;
+    } else {
+        for (auto& c : all) {
+            if (!b->own_shape) {
+                if (c.block == 256) continue;
+                c.block = given;
+            }
+            const int rc = set_shape(b, vec, c.block, c.fused);
+            if (rc != LBM_OK) return rc;
+            c.worth = shape_us(b, check_every) * (c.block == 256 ? (b->n > b->sms ? 1.06 : 1.035) : 1.0);
+            if (c.worth < best.worth) best = c;
+        }
+    }
+    const int rc = set_shape(b, vec, best.block, best.fused);
+    if (rc != LBM_OK) return rc;
+    b->shape_check = check_every;
+    // (in the order of the stream, so after the runs before)
+    LBM_BCK(b, cudaMemcpyAsync(b->d_inst, b->inst.data(), sizeof(BatchInstance) * b->n, cudaMemcpyHostToDevice, b->stream));
+    return LBM_OK;
+}
+// A shape asked for: its kernel of the check interval in use.
+int ask_shape(lbm_batch* b, int vec, int block) {
+    if (!pick_batch_kernel(b->storage, vec, block, false))
+        return berr(b, LBM_ERR_UNSUPPORTED, "no batch kernel with vec=%d block=%d for this storage", vec, block);
+    const int check = b->shape_check < 0 ? 100 : b->shape_check;
+    b->own_shape = false;
+    b->vec = vec;
+    b->block = block;
+    if (b->storage == LBM_F64) return set_shape(b, vec, block, false);
+    b->shape_check = -1;
+    return choose_shape(b, check);
+}
 // Equilibrium initialisation of every instance from concatenated dense fields.
 template <typename S>
 __global__ void batch_init_kernel(S* slab, const BatchInstance* __restrict__ inst, const BatchState* __restrict__ st,
@@ -192,7 +330,7 @@ int record_run(lbm_batch* b, long long target, int check_every, double growth) {
         int ce = check_every;
         double gr = growth;
         void* args[] = {&slab, &di, &ds, &dord, &n, &dq, &tg, &ce, &gr};
-        cudaLaunchKernel(b->kernel, dim3(b->grid), dim3(b->block), args, batch_smem(b->storage, b->block), cap);
+        cudaLaunchKernel(b->kernel, dim3(b->grid), dim3(b->block), args, b->smem, cap);
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(cap, &graph);
         if (e == cudaSuccess) {
@@ -255,7 +393,7 @@ int lbm_batch_create(lbm_batch** out, int n, const lbm_instance_desc* desc, int 
         I.a.kread = d.model == LBM_K_PRE ? 1 : (d.model == LBM_K_EQ ? 2 : 0);
         lbm::fill_consts(I.a);
         I.model = (d.model == LBM_K_PRE || d.model == LBM_K_EQ) ? LBM_K : d.model;
-        I.pad = 0;
+        I.march_from = lbm::kNeverMarch;
         I.ke_ref = d.ke_ref;
         I.ke_factor = d.ke_factor;
         I.eq = lbm::equilibrium_consts(d.ux_ref, d.uy_ref);
@@ -300,11 +438,9 @@ int lbm_batch_create(lbm_batch** out, int n, const lbm_instance_desc* desc, int 
         rc = e == cudaErrorMemoryAllocation ? LBM_ERR_NOMEM : LBM_ERR_CUDA;
     } else {
         rc = reset_states(b);
-        if (rc == LBM_OK) {
-            int vec, block;
-            default_shape(storage, &vec, &block);
-            rc = set_shape(b, vec, block);
-        }
+        b->order = order;
+        for (const BatchInstance& I : inst) b->models = b->models || I.model != inst[0].model;
+        if (rc == LBM_OK) rc = choose_shape(b, 100);
     }
     if (rc != LBM_OK) {
         lbm_batch_destroy(b);
@@ -361,7 +497,9 @@ int lbm_batch_run(lbm_batch* b, long long target_steps, int check_every, double 
     if (!b) return LBM_ERR_INVALID_ARG;
     if (target_steps < 0 || check_every < 0 || !(growth > 1.0) || !std::isfinite(growth))
         return berr(b, LBM_ERR_INVALID_ARG, "invalid run parameters");
-    int rc = record_run(b, target_steps, check_every, growth);
+    int rc = choose_shape(b, check_every);
+    if (rc) return rc;
+    rc = record_run(b, target_steps, check_every, growth);
     if (rc) return rc;
     LBM_BCK(b, cudaGraphLaunch(b->exec, b->stream));
     return LBM_OK;
@@ -415,7 +553,7 @@ int lbm_batch_get_populations(lbm_batch* b, int index, double* f) {
 
 int lbm_batch_set_shape(lbm_batch* b, int vec, int block) {
     if (!b) return LBM_ERR_INVALID_ARG;
-    return set_shape(b, vec, block);
+    return ask_shape(b, vec, block);
 }
 
 int lbm_batch_get_shape(const lbm_batch* b, int* vec, int* block, int* grid) {
@@ -447,8 +585,8 @@ int lbm_batch_autotune(lbm_batch* b, long long trial_steps, int check_every, int
     int rc = LBM_OK;
     for (const auto& c : cand) {
         if (e != cudaSuccess) break;
-        if (!pick_batch_kernel(b->storage, c[0], c[1])) continue;
-        if (set_shape(b, c[0], c[1]) != LBM_OK) continue;
+        if (!pick_batch_kernel(b->storage, c[0], c[1], false)) continue;
+        if (ask_shape(b, c[0], c[1]) != LBM_OK || choose_shape(b, check_every) != LBM_OK) continue;
         rc = record_run(b, start + trial_steps, check_every, 1e4);
         if (rc != LBM_OK) break;
         cudaEventRecord(e0, b->stream);
@@ -468,7 +606,7 @@ int lbm_batch_autotune(lbm_batch* b, long long trial_steps, int check_every, int
     cudaFree(saved);
     if (rc != LBM_OK) return rc;
     if (e != cudaSuccess) return berr(b, LBM_ERR_CUDA, "autotune: %s", cudaGetErrorString(e));
-    rc = set_shape(b, best_v, best_b);
+    rc = ask_shape(b, best_v, best_b);
     if (rc) return rc;
     if (vec) *vec = best_v;
     if (block) *block = best_b;

@@ -4,13 +4,14 @@
 #include "lbm_internal.h"
 
 namespace lbm {
-const void* batch_kernel_f32(int vec, int block) {
-    if (vec == 4 && block == 256) return (const void*)batch_kernel<float, 4, 256>;
-    if (vec == 4 && block == 128) return (const void*)batch_kernel<float, 4, 128>;
-    if (vec == 4 && block == 512) return (const void*)batch_kernel<float, 4, 512>;
-    if (vec == 2 && block == 256) return (const void*)batch_kernel<float, 2, 256>;
-    if (vec == 2 && block == 128) return (const void*)batch_kernel<float, 2, 128>;
-    if (vec == 2 && block == 512) return (const void*)batch_kernel<float, 2, 512>;
+const void* batch_kernel_f32(int vec, int block, bool fused) {
+    if (!fused) return batch_kernel_f32_steps(vec, block);
+    if (vec == 4 && block == 256) return (const void*)batch_kernel<float, 4, 256, true>;
+    if (vec == 4 && block == 128) return (const void*)batch_kernel<float, 4, 128, true>;
+    if (vec == 4 && block == 512) return (const void*)batch_kernel<float, 4, 512, true>;
+    if (vec == 2 && block == 256) return (const void*)batch_kernel<float, 2, 256, true>;
+    if (vec == 2 && block == 128) return (const void*)batch_kernel<float, 2, 128, true>;
+    if (vec == 2 && block == 512) return (const void*)batch_kernel<float, 2, 512, true>;
     return nullptr;
 }
 }  // namespace lbm

@@ -5,7 +5,7 @@
 
 namespace lbm {
 const void* batch_kernel_f64(int vec, int block) {
-    if (vec == 2 && block == 256) return (const void*)batch_kernel<double, 2, 256>;
+    if (vec == 2 && block == 256) return (const void*)batch_kernel<double, 2, 256, false>;
     return nullptr;
 }
 }  // namespace lbm

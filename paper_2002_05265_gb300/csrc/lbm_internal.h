@@ -40,11 +40,15 @@ const void* march_kernel_f32(bool shifted, bool pairs, bool roll);
 const void* march_kernel_f16(bool shifted, bool pairs, bool roll);
 const void* march_kernel_bf16(bool shifted, bool pairs, bool roll);
 
-// Batched persistent sweep kernel for (vector width, CTA size); nullptr if not instantiated.
+// Batched persistent sweep kernel for (vector width, CTA size), with the time-fused marches or (steps)
+// without; nullptr if not instantiated.
 const void* batch_kernel_f64(int vec, int block);
-const void* batch_kernel_f32(int vec, int block);
-const void* batch_kernel_f16(int vec, int block);
-const void* batch_kernel_bf16(int vec, int block);
+const void* batch_kernel_f32(int vec, int block, bool fused);
+const void* batch_kernel_f32_steps(int vec, int block);
+const void* batch_kernel_f16(int vec, int block, bool fused);
+const void* batch_kernel_f16_steps(int vec, int block);
+const void* batch_kernel_bf16(int vec, int block, bool fused);
+const void* batch_kernel_bf16_steps(int vec, int block);
 
 // CTA size for a grid-stride kernel of so many threads: 256, or less where two CTAs per SM would not
 // be filled, down to a warp.
