@@ -513,9 +513,10 @@ int tile_steps_per_launch(const lbm_group* g) {
     return (int)std::min<long long>(std::min<long long>(per, cap), LBM_TILE_STEPS_PER_LAUNCH);
 }
 
-// FP32 operations of one node update, by model (lbm_device.cuh)
+// Operations of collide_f32 for one node, by model: what a march's time goes by (K : BGK 1.29; measured
+// at 16384^2 1157 : 963 us, 1.20)
 int march_cost(int model) {
-    static const int cost[] = {60, 66, 68, 79, 81, 85, 65, 75};
+    static const int cost[] = {80, 80, 83, 96, 98, 103, 81, 93};
     return cost[kernel_model(model)];
 }
 
@@ -552,6 +553,17 @@ long long march_ctas(const lbm_group* g, const MarchPlan& p, double work) {
     for (const lbm_ctx* c : g->ctx)
         ctas += ((long long)((c->nx + width - 1) / width) * march_bands(c, p, work) + p.per - 1) / p.per;
     return ctas;
+}
+
+// What shares the plan's marches out to the lattices: their work, or a little more where the lattices'
+// last CTAs, each rounded up, would be some more than the plan's (two 512^2 lattices, BGK and K: 153 CTAs
+// for 152 SMs 6.9 us a step, 152 5.0).
+double march_shares(const lbm_group* g, const MarchPlan& p) {
+    const double work = march_work(g, p.t);
+    double more = work;
+    for (int k = 0; k < 32; ++k, more *= 1.01)
+        if (march_ctas(g, p, more) <= p.warps / p.per) return more;
+    return work;
 }
 
 // Large lattices fuse as many steps as the kernel has levels, in whole waves of resident warps
@@ -601,7 +613,7 @@ MarchPlan march_plan(const lbm_group* g, long long n) {
 // the shift and the models' operations as measured (14 and 15 columns, 300,000 rows, K: FP32 75.4 and
 // 85.7 us a step, FP16 78.5 and 98.3; 4096^2 K FP32 77 us, with shift 91).
 double march_us(const lbm_group* g, const MarchPlan& p) {
-    const double work = march_work(g, p.t);
+    const double work = march_shares(g, p);
     const long long ctas = march_ctas(g, p, work);
     int rows = 1, odd = 0;
     double nodes = 0.0, cost = 0.0;
@@ -667,7 +679,7 @@ int launch_march(lbm_group* g, cudaStream_t s, int t, const MarchPlan& p) {
     ma.n = (int)g->ctx.size();
     ma.t = t;
     const int width = lbm::march_width(t);
-    const double work = march_work(g, t);
+    const double work = march_shares(g, {t, p.warps, p.per});
     unsigned begin = 0;
     int rows = 1;
     for (size_t k = 0; k < g->ctx.size(); ++k) {
@@ -1360,7 +1372,7 @@ int lbm_group_create(lbm_group** out, lbm_ctx* const* ctxs, int n, int graph_ste
     // equilibrium, unless a context asks for a kernel family, form or launch shape.  (FP64 is bound
     // by its pipe with one step a launch already.)  Groups of several models take the rolled form,
     // whose code for four models at a time stays in an SM's instruction cache (eight 1024^2
-    // lattices of all models 42 us a step, unrolled 59; one model: 16384^2 K 1068, unrolled 1042)
+    // lattices of all models 42.1 us a step, unrolled 47.5; one model: 16384^2 K 1228, unrolled 1156)
     bool march = n <= lbm::kGroupMax && ctxs[0]->storage != LBM_F64;
     bool pairs = true, mixed = false;
     for (int k = 0; k < n; ++k) {
