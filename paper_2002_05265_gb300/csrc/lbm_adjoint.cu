@@ -38,8 +38,8 @@ constexpr int kAdjBlock = 256;
 template <typename S> constexpr int kAdjMinBlocks = sizeof(S) == 8 ? 0 : LBM_ADJ_MIN_BLOCKS;
 
 // Nodes per thread of the adjoint step: it holds the populations and the adjoints of every
-// node it handles, so it uses half the vector width of the forward kernel (FP32: 2 nodes,
-// FP64: 1 node) to keep its registers, and so its occupancy, close to the forward kernel's.
+// node it handles, so in FP32 it uses half the vector width of the forward kernel (2 nodes;
+// FP64: 1 node, as the forward kernel) to keep its registers, and so its occupancy, close to it.
 #ifndef LBM_ADJ_VEC_DIV
 #define LBM_ADJ_VEC_DIV 2
 #endif

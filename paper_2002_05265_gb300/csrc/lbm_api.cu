@@ -1304,7 +1304,9 @@ int lbm_group_create(lbm_group** out, lbm_ctx* const* ctxs, int n, int graph_ste
         // that the wide form leaves a single lattice to the general form's wavefront launches
         // where those apply (measured, FP32: 4096^2 0.96 of the copy bandwidth in the wavefront
         // against 0.91 in the wide form; 8192^2 wide 0.96 against 0.94 for the general form's
-        // one-step launches); otherwise the general form.
+        // one-step launches); otherwise the general form.  (Runs of several steps with every choice
+        // left open take the time-fused launches instead, so there the rule decides a single step,
+        // where the general form has no wavefront: 4096^2 K 200 us, in the wide form 197.)
         const bool light = storage != LBM_F64 && light_models(ctxs, n);
         const int one_form = storage == LBM_F64 ? -1 : ((light && storage != LBM_BF16) ? 1 : 2);
         const lbm_ctx* c0 = ctxs[0];
@@ -1572,9 +1574,9 @@ int lbm_adjoint_run(lbm_ctx* c, long long nsteps, int loss, const double* ux_tar
         if (rc != LBM_OK) break;
     }
     LBM_ADJ(cudaEventRecord(ev[1], c->stream));
-    // the recomputation takes the forward run's kernel family (the context's own group); with
-    // the register-staged kernels each adjoint launch also recomputes a step of the next
-    // segment into a second ring (fused launches)
+    // the recomputation takes the one-step kernels of the context's own group, whose bits the forward
+    // run's time-fused launches have too; with the register-staged kernels each adjoint launch also
+    // recomputes a step of the next segment into a second ring (fused launches)
     lbm_group* fg = (c->own_group && c->own_group->tiled) ? c->own_group : nullptr;
     const bool fused = !fg && plan.grid_fused > 0 && nseg > 1 && K > 1;
     LBM_ADJ(cudaMalloc(&ring, (size_t)(fused ? 2 : 1) * K * bufb));

@@ -146,7 +146,7 @@ template <typename S> struct DefaultVec {
 // Nodes per thread of the register-staged step kernels: the default, but one for FP64, where a
 // scheduler takes 64 clocks for an instruction of one warp (measured, whatever lanes are active): what
 // counts there is that every scheduler has one.  With CTAs to match (spread_block) a step of 128 x 128
-// BGK takes 5.5 us instead of 11.0, 67 x 37 CHM 4.3 us instead of 16.4.
+// BGK takes 4.0 us instead of 11.0, 67 x 37 CHM 4.3 us instead of 16.4.
 template <typename S> struct StepVec {
     static constexpr int value = sizeof(S) == 8 ? 1 : DefaultVec<S>::value;
 };
@@ -514,8 +514,9 @@ __device__ __forceinline__ void collide_f64(const double (&g)[9], double (&o)[9]
 // so that every kernel form and both widths give the same bits; 16-bit storage needs that most: one
 // population rounded the other way spreads until, after some hundred steps, two BF16 runs differ by
 // as much as either does from FP64.  Products that a sum takes up fused are not formed again.
-// Operations of one node: BGK 80, K 103 (the expressions of collide_f64 would be 60 and 85 and the
-// time-fused kernel 8-11 % faster, 1042 us against 1157 a step of 16384^2 K; they round differently).
+// Operations of one node: BGK 80, K 103 (the expressions of collide_f64 would be 60 and 85, the
+// reciprocal's two included, and the time-fused kernel 8-11 % faster, 1042 us against 1157 a step of
+// 16384^2 K; they round differently).
 template <int MODEL, typename P, bool SHIFT>
 __device__ __forceinline__ void collide_f32(const P (&g)[9], P (&o)[9], const Consts<P>& c, P& rho_out, P& ux_out,
                                             P& uy_out) {

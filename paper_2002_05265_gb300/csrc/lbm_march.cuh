@@ -3,10 +3,12 @@
 //
 // A warp owns a strip of 64 columns, two neighbouring nodes per lane, and marches up the rows.
 // At each row it loads the nine pulled rows, collides them (level 1, time step 1), keeps what
-// level 2 will pull, collides row y - 1 of level 2 from that, and so on; level t is stored.  A level needs the rows y - 1, y, y + 1 of the level below: the populations with
-// xi_y = -1 come from the row that level just produced, those with xi_y = 0 and +1 from one
-// and two rows earlier, so nine pairs per level wait in the lane's own column of shared memory (or
-// three of them in registers).  The neighbours in x are lanes: one shuffle per x-shifted population.  Warps share nothing, so there is no barrier.
+// level 2 will pull, collides row y - 1 of level 2 from that, and so on; level t is stored.  A level
+// needs the rows y - 1, y, y + 1 of the level below: the populations with xi_y = -1 come from the row
+// that level just produced, those with xi_y = 0 and +1 from one and two rows earlier, so nine pairs
+// per level wait in the lane's own column of shared memory (or three of them in registers).  The
+// neighbours in x are lanes: one shuffle per x-shifted population.  Warps share nothing, so there is
+// no barrier.
 // The price is redundant work at the strip's edges: every level spoils one node on each side
 // (the outer lanes' results are discarded, adjacent strips overlap: 56 of 64 columns are stored at
 // t = 4), and a march over H rows starts with rows of the lower levels that its neighbour in y also
@@ -19,7 +21,8 @@
 // instructions), reached by colliding the lane's two nodes with the two-wide FP32 instructions.
 // Measured, us a step, one-step launches before and four-step launches after: 16384^2 FP32 K 2905 ->
 // 1157, BGK 2824 -> 963; 4096^2 CHM 184 -> 74, BF16 116 -> 76; 2048^2 CM 48.8 -> 20.9; 1024^2 K 10.0 ->
-// 7.2; eight 1024^2 lattices of all models 93 -> 42.5.
+// 7.1; eight 1024^2 lattices of all models 93 -> 42.1.
+// A reference velocity (SHIFT) costs 18 %: 4096^2 K 77.2 us a step without, 90.9 with.
 // Fewer or more levels: 3 at most 1.33x the time of 4 (4096^2 BGK), 5 1.05x, 6 1.2x (the edges).
 #pragma once
 
@@ -105,19 +108,10 @@ template <typename S> __device__ __forceinline__ void pair_close(Pair16<S>& p, F
 }
 
 constexpr int kMarchWarps = 8;    // most warps of a CTA; all of one lattice
-#ifndef LBM_MARCH_T32
-#define LBM_MARCH_T32 4
-#endif
-#ifndef LBM_MARCH_T16
-#define LBM_MARCH_T16 4
-#endif
-#ifndef LBM_MARCH_MINB
-#define LBM_MARCH_MINB 2
-#endif
 // Most time steps of a launch, and the CTAs of kMarchWarps warps per SM the registers are sized for.
 template <typename S> struct MarchForm {
-    static constexpr int TMAX = sizeof(S) == 4 ? LBM_MARCH_T32 : LBM_MARCH_T16;
-    static constexpr int MINB = LBM_MARCH_MINB;
+    static constexpr int TMAX = 4;
+    static constexpr int MINB = 2;
 };
 constexpr int kMarchSpan = 64;    // columns of a strip, discarded edges included
 __host__ __device__ constexpr int march_edge(int t) { return (t + 1) / 2; }             // discarded lanes a side
