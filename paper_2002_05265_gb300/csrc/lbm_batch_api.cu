@@ -45,6 +45,7 @@ struct lbm_batch {
     bool own_shape = true;             // the shape is the library's choice
     int shape_check = -1;              // check interval the kernel was chosen for
     std::vector<int> order;            // largest instances first
+    std::vector<int> bands;            // of a march, by instance
     const void* kernel = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long g_target = -1;
@@ -100,8 +101,8 @@ double one_step_us(const BatchInstance& I, int vec, int block, int resident, boo
     const double alone = 0.7 + nodes / (block >= 512 ? 1020.0 : (block >= 256 ? 850.0 : 630.0));
     return std::max(alone, 0.8 + nodes * resident / (spill ? 630.0 : 1040.0));
 }
-// t steps fused, a step: rounds of the CTA's warps over strips and bands, as batch_march takes them.
-double fused_us(const BatchInstance& I, int block, int resident, int t) {
+// Bands of a marching instance, as batch_march picks them.
+int fused_bands(const BatchInstance& I, int block) {
     const int warps = block / 32, most = lbm::MarchForm<float>::TMAX;
     const int strips = (I.a.nx + lbm::march_width(most) - 1) / lbm::march_width(most);
     long long least = 1ll << 40;
@@ -113,6 +114,11 @@ double fused_us(const BatchInstance& I, int block, int resident, int t) {
             bands = b;
         }
     }
+    return bands;
+}
+// t steps fused, a step: rounds of the CTA's warps over strips and bands.
+double fused_us(const BatchInstance& I, int bands, int block, int resident, int t) {
+    const int warps = block / 32;
     const long long tasks = (long long)((I.a.nx + lbm::march_width(t) - 1) / lbm::march_width(t)) * bands;
     const double rows = (double)((tasks + warps - 1) / warps) * ((I.a.ny + bands - 1) / bands + t - 1);
     const int load = warps * resident;   // warps of the SM: a level row takes so long
@@ -143,11 +149,11 @@ double sweep_us(const lbm_batch* b, const BatchInstance& I) {
 }
 // Least check interval from which marching instance I is quicker (kNeverMarch: never): the fewest
 // steps t that pay fused are what lies between two checks.
-int march_from(const lbm_batch* b, const BatchInstance& I) {
-    int from = lbm::kNeverMarch;
-    if (!b->fused) return from;
+int march_from(const lbm_batch* b, const BatchInstance& I, int bands) {
     const double one = sweep_us(b, I);
-    for (int t = lbm::MarchForm<float>::TMAX; t >= 1 && fused_us(I, b->block, resident_ctas(b), t) < one; --t) from = t + 1;
+    int from = lbm::kNeverMarch;
+    for (int t = lbm::MarchForm<float>::TMAX; t >= 1 && fused_us(I, bands, b->block, resident_ctas(b), t) < one; --t)
+        from = t + 1;
     return from;
 }
 
@@ -179,7 +185,12 @@ int set_shape(lbm_batch* b, int vec, int block, bool fused) {
     b->per_sm = per_sm;
     // resident CTAs only (a persistent grid); never more CTAs than instances
     b->grid = std::min(b->sms * per_sm, b->n);
-    for (BatchInstance& I : b->inst) I.march_from = march_from(b, I);
+    b->bands.resize(b->n);
+    for (int i = 0; i < b->n; ++i) {
+        BatchInstance& I = b->inst[i];
+        b->bands[i] = fused ? fused_bands(I, block) : 1;
+        I.march_from = fused ? march_from(b, I, b->bands[i]) : lbm::kNeverMarch;
+    }
     return LBM_OK;
 }
 
@@ -194,7 +205,7 @@ double shape_us(const lbm_batch* b, int check_every) {
     for (int i : b->order) {
         const BatchInstance& I = b->inst[i];
         const double one = sweep_us(b, I);
-        const double rest = lbm::batch_fused(I.march_from, check_every) ? fused_us(I, b->block, resident, t) : one;
+        const double rest = lbm::batch_fused(I.march_from, check_every) ? fused_us(I, b->bands[i], b->block, resident, t) : one;
         double us = rest + (one - rest + check_us(I, b->block, resident)) / apart;
         if ((int)busy.size() == b->grid) {
             us += busy.top();
