@@ -562,7 +562,7 @@ double march_shares(const lbm_group* g, const MarchPlan& p) {
     const double work = march_work(g, p.t);
     double more = work;
     for (int k = 0; k < 32; ++k, more *= 1.01)
-        if (march_ctas(g, p, more) <= p.warps / p.per) return more;
+        if (march_ctas(g, p, more) <= (p.warps + p.per - 1) / p.per) return more;
     return work;
 }
 
