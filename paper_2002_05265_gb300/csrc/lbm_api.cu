@@ -581,11 +581,11 @@ MarchPlan march_plan(const lbm_group* g, long long n) {
     int most = (int)std::min<long long>(g->march, n);
     long long rows = march_strip_rows(g, most);
     if (most == g->march && rows >= 24 * slots) {
-        // two steps a launch, whose strips are 60 columns wide, where that saves a strip worth more than
-        // the second half of the fusion (57-60 columns: 500,000 rows in BF16 296 -> 218 us, 100,000 in
-        // FP32 56 -> 52; 2048^2: FP32 27.5 against 21.4, FP16 23.8 against 22.2)
-        const double dearer = g->ctx[0]->storage == LBM_F32 ? 1.55 : 1.13;
-        if (dearer * (double)march_strip_rows(g, 2) < (double)rows) rows = march_strip_rows(g, most = 2);
+        // 16-bit lattices: two steps a launch, whose strips are 60 columns wide, where that saves a strip
+        // worth more than the second half of the fusion (57 x 500,000 BF16 296 -> 218 us; 2048^2 FP16
+        // 23.8 against 22.2; in FP32, 27.5 against 21.4 there, it never is)
+        if (g->ctx[0]->storage != LBM_F32 && 1.13 * (double)march_strip_rows(g, 2) < (double)rows)
+            rows = march_strip_rows(g, most = 2);
         long long waves = (rows + 160 * slots - 1) / (160 * slots);
         if (g->mixed && waves < 2 && rows >= 48 * slots) waves = 2;
         return {most, slots * waves, lbm::kMarchWarps};
@@ -615,12 +615,13 @@ MarchPlan march_plan(const lbm_group* g, long long n) {
 double march_us(const lbm_group* g, const MarchPlan& p) {
     const double work = march_shares(g, p);
     const long long ctas = march_ctas(g, p, work);
-    int rows = 1, odd = 0;
+    int rows = 1, odd = 0, narrow = 1 << 30;
     double nodes = 0.0, cost = 0.0;
     for (const lbm_ctx* c : g->ctx) {
         const int bands = march_bands(c, p, work);
         rows = std::max(rows, (c->ny + bands - 1) / bands);
         odd |= c->nx & 1;
+        narrow = std::min(narrow, c->nx);
         nodes += (double)c->nx * c->ny;
         cost += (double)c->nx * c->ny * march_cost(c->model);
     }
@@ -629,7 +630,7 @@ double march_us(const lbm_group* g, const MarchPlan& p) {
     const double waves = std::max(1.0, (double)ctas / ((double)g->sms * room));
     const double each = load <= 1 ? 0.25 : (load <= 2 ? 0.14 + 0.11 * load : 0.36 + (load - 2) * (0.06 + 0.24 / p.t));
     const int storage = g->ctx[0]->storage;
-    double f = odd ? (storage == LBM_F32 ? 1.12 : (storage == LBM_F16 ? 1.33 : 1.25)) : 1.02;
+    double f = odd ? (storage == LBM_F32 ? 1.12 + 0.75 / narrow : (storage == LBM_F16 ? 1.33 : 1.25)) : 1.02;
     f *= 0.5 + 0.5 * cost / (nodes * march_cost(LBM_K));
     if (tile_shift(g) == 1) f *= 1.1;
     return f * (2.2 + each * p.t * (rows + p.t - 1) * waves) / p.t;
