@@ -301,14 +301,16 @@ cudaError_t launch_kernel(const void* kernel, int grid, int block, int smem, voi
 // Whether register-staged steps overlap their launches.  What it saves is the launch latency; what it
 // costs is the even spread of the CTAs over the SMs, since those of the next launch take the places
 // as they come free.  Two launches of a warp for every second scheduler fit side by side (67 x 37 FP64
-// BGK 3.46 against 3.65 us a step, recorded; launched one by one a few more do, 100^2 4.6 against 6.2); more warps in recorded steps, whose latency is short, lose
-// by it (FP64 BGK 128^2 5.51 against 3.97 us, 256^2 of second order 38 against 20.6, FP16 1001 x 777 7.6
-// against 6.2), and FP64 steps, which wait for the busiest scheduler's pipe, lose launched one by one
-// too (160^2 14.5 against 7.5); FP32 and 16-bit steps launched one by one gain (512^2 4.7 against 6.2,
-// 1001 x 777 K 7.9 against 8.5), unless a warp takes several rows (3 x 30,000 FP32 17 against 8).
+// BGK 3.46 against 3.65 us a step, recorded; launched one by one a few more do, 100^2 4.6 against
+// 6.2); more warps in recorded steps, whose latency is short, lose by it (FP64 BGK 128^2 5.51 against
+// 3.97 us, 256^2 of second order 38 against 20.6, FP16 1001 x 777 7.6 against 6.2), and FP64 steps,
+// which wait for the busiest scheduler's pipe, lose launched one by one too (160^2 14.5 against 7.5);
+// FP32 and 16-bit steps launched one by one gain (512^2 4.7 against 6.2, 1001 x 777 K 7.9 against 8.5,
+// 57 x 1000 2.8 against 4.1, 17 x 30,000 FP16 8.0 against 10.3), unless a row is a few vectors (3 x
+// 30,000 FP32 17 against 8, 13 x 30,000 9.3 against 8.2).
 bool overlap_steps(int storage, int grid, int block, int nseg, bool recorded) {
     const long long warps = (long long)grid * block / 32;
-    return warps <= (recorded ? 304 : 400) || (!recorded && storage != LBM_F64 && nseg >= 32);
+    return warps <= (recorded ? 304 : 400) || (!recorded && storage != LBM_F64 && nseg >= (storage == LBM_F32 ? 5 : 3));
 }
 
 int launch_step_once(lbm_ctx* c, cudaStream_t s, bool recorded) {
