@@ -194,6 +194,12 @@ class ClockSampler:
                 "power_w_max": float(max(power)) if power else None, "reasons": sorted(reasons)}
 
 
+# FP32 operations of one node's collision by model (collide_f32 in csrc/lbm_device.cuh; a fused pair is
+# one) and their rate on GB300, half the FLOP rate of a measured FMA loop
+FP32_OPS = {"bgk": 80, "rm": 80, "hm": 83, "cm": 96, "chm": 98, "k": 103, "pr": 81, "rr": 93}
+FP32_PEAK_TOPS = 36.8
+
+
 def measured_peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(path):
@@ -516,7 +522,7 @@ def bench_config(S, world):
                         f"8 collision models (BGK, RM, HM, CM, CHM, K, PR, RR), FP32 shifted storage",
             "lattices": len(MODELS), "lattice": f"{L}x{L}", "sim_steps": S,
             "check_every": CHECK_EVERY, "graph_steps": GRAPH_STEPS,
-            "l2": "inputs larger than L2: 8 lattices x 75.5 MB advanced in turn each time step",
+            "l2": "inputs larger than L2: 8 lattices x 75.5 MB advanced together",
             "parallelism": f"replicas x{world}" if world > 1 else "single GPU"}
 
 
@@ -1060,9 +1066,11 @@ def main():
     avg_launch_s = replay_ms / 1e3 / kernel_launches
     fused = lattice_steps / kernel_launches / len(MODELS)
     desc = lbm.lbm_group_describe(group)
-    # every choice left to the library: fused launches (lbm_group_describe tells the one-step form)
-    marched = (fused > 1 and args.path == "auto" and args.form == "auto" and args.order == "auto" and
-               not args.stages and not args.launch_steps)
+    # every choice left to the library, and launches of as many steps as neither the one-step kernels
+    # nor a whole replay in one copy-engine launch would have: time-fused launches
+    # (lbm_group_describe tells the one-step form)
+    marched = (args.path == "auto" and args.form == "auto" and args.order == "auto" and not args.stages and
+               not args.launch_steps and fused > 1 and fused != min(desc["steps_per_launch"], GRAPH_STEPS))
     # launches of the copy-engine kernel with several steps move the populations at every step
     bytes_per_launch = BYTES_PER_LU["f32"] * L * L * len(MODELS) * (1 if marched else fused)
     achieved = bytes_per_launch / avg_launch_s / 1e9
@@ -1077,8 +1085,13 @@ def main():
         kname = f"lbm::tile_step_kernel<float> (cp.async.bulk ring, {form} form)"
     else:
         kname = "lbm::group_step_kernel<float> (register-staged)"
-    roofline = {"bound": "fp32" if marched else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": traffic, "peak_source": peak_kind,
+    hbm = {"achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_kind}
+    bound = {"bound": "hbm", **hbm}
+    if marched:   # operations of the collisions as the FP32 pipe takes them, a fused pair as one
+        rate = sum(FP32_OPS.values()) * L * L * fused / avg_launch_s / 1e12
+        bound = {"bound": "fp32", "achieved": rate, "peak": FP32_PEAK_TOPS, "unit": "Top/s",
+                 "frac": rate / FP32_PEAK_TOPS, "peak_source": "measured (FMA loop, 73.6 TFLOP/s)", "hbm": hbm}
+    roofline = {**bound, "traffic": traffic,
                 "launch_us": avg_launch_s * 1e6, "bytes_per_launch": bytes_per_launch, "steps_per_launch": fused,
                 "one_step_floor_us": BYTES_PER_LU["f32"] * L * L * len(MODELS) / peak / 1e3,
                 "step_us": avg_launch_s * 1e6 / fused,

@@ -245,7 +245,8 @@ int lbm_get_layout(const lbm_ctx* ctx, int* pitch, int* grid, int* block);
  *   LBM_PATH_AUTO    (the default) runs of two or more steps of 32- or 16-bit lattices with the
  *                    extended equilibrium take time-fused launches, each of which advances up to
  *                    four steps with one read and one write of the populations (unless stages, a
- *                    launch shape or a tile form is asked for); every other step BULK where the
+ *                    launch shape or a tile form is asked for, or the lattices are so narrow, flat or
+ *                    odd that VECTOR is quicker); every other step BULK where the
  *                    row length allows it and a time step has at least one tile per resident CTA,
  *                    else VECTOR.  The arithmetic of a node is the same, bit for bit.
  * Applies to the context's next lbm_step and to groups created afterwards.  Errors:
@@ -390,8 +391,10 @@ int lbm_batch_run(lbm_batch* b, long long target_steps, int check_every, double 
 int lbm_batch_status(lbm_batch* b, int* status, long long* blowup_step, long long* steps, double* diag4);
 /* Canonical pre-collision populations of one instance as FP64 [9][ny][nx]. */
 int lbm_batch_get_populations(lbm_batch* b, int index, double* f);
-/* Kernel shape: `vec` x-nodes per thread (of the steps that check, and of FP64) and `block` threads
- * per CTA (one CTA advances an instance; by default 512, FP64 256).  autotune times every
+/* Kernel shape: `vec` x-nodes per thread (of steps taken one at a time) and `block` threads per CTA
+ * (one CTA advances an instance; by default 512 or 256, FP64 256, chosen from the instances and the
+ * check interval of a run, for 100 until then).  Whether an instance's steps between two checks are
+ * fused is chosen for the shape and the check interval.  autotune times every
  * instantiated shape for `trial_steps` steps from the current state (restoring the state
  * after each trial), keeps the fastest and reports it. */
 int lbm_batch_set_shape(lbm_batch* b, int vec, int block);
